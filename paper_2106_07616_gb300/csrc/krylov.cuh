@@ -2,6 +2,7 @@
 #pragma once
 #include "amg.cuh"
 #include "common.cuh"
+#include "resident.cuh"
 
 namespace rbffd {
 
@@ -72,6 +73,10 @@ struct MixedArgs {
   double inner_tol;      // relative reduction asked of each inner solve
   int inner_maxit;       // cap on inner iterations per sweep
   int max_sweeps;
+  // resident solve (resident.cuh): the team and its halo lists (nb = 0: none),
+  // and the vectors published to the other CTAs, n x NR values side by side
+  ResPlan res;
+  void *pubt, *pubv;
 };
 
 int krylov_max_blocks(rbffd_ctx *ctx, int nr);

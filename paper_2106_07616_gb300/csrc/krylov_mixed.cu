@@ -21,6 +21,7 @@
 #include "krylov.cuh"
 #include "inner_arith.cuh"
 #include "krylov_dev.cuh"
+#include "resident.cuh"
 
 namespace rbffd {
 
@@ -574,6 +575,492 @@ __global__ void __launch_bounds__(NT) k_bicgstab_ir(MixedArgs A) {
   bicgstab_ir_body<NR, NT, IA>(A, blockIdx.x, gridDim.x);
 }
 
+// ---- the resident solve (resident.cuh) --------------------------------------
+//
+// The same sweeps and the same inner BiCGSTAB as bicgstab_ir_body, two team
+// exchanges per inner iteration, with everything but one vector a phase on
+// chip: the matrix in registers (E entries a lane), and for every entry of
+// the CTA's halo list the residual / s, p, v and the inverse diagonal in
+// shared memory.  Every CTA advances the recurrences of its whole halo with
+// the same operations as their owners, so neighbours only need
+//   phase A: t of the previous iteration (r = s - omega t and
+//            p = r + beta (p - omega v) follow on the spot),
+//   phase C: v of this one (s = r - alpha v follows),
+// one load an entry of the list instead of up to five a matrix entry or
+// window entry.  What bounds it: the exchange (about 1.2 us over the grid,
+// twice an iteration) and the halo's round trip.
+// Measured on GB300, a whole outer iteration with the streaming solve and
+// with this one (the p' solve the same): cavity 200^2 (q = 30, two right-hand
+// sides) 12.5 -> 8.4 ms, cylinder 147 827 (q = 20, two single solves)
+// 20.2 -> 11.6 ms, Kovasznay 50^2 (one cluster) 6.9 -> 4.9 ms.
+namespace {
+
+template <int NR, class IA>
+struct IrCoef {
+  typename IA::C alp[NR], omg[NR], nomg[NR], bet[NR], nalp[NR];
+  int run[NR], fin[NR], any;
+};
+
+template <int NR, class IA, int E>
+__global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
+  using S = typename IA::S;
+  using PT = typename IA::P;
+  using V = res::Vec<S, NR>;
+  constexpr int ES = (int)sizeof(V);
+  __shared__ PT wsum[5 * NR * 32];
+  __shared__ PT cpart[2 * 5 * NR * RES_CLUSTER];
+  __shared__ double wsum64[2 * NR * 32], cpart64[2 * 2 * NR * RES_CLUSTER];
+  __shared__ PT tot[5 * NR];
+  __shared__ double tot64[2 * NR];
+  __shared__ IRS ks[NR];
+  __shared__ double lim2[NR], big2[NR];  // (inner_tol r0)^2, (1e3 r0)^2 of the sweep
+  __shared__ IrCoef<NR, IA> co;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int lb = blockIdx.x, nb = gridDim.x, tid = threadIdx.x;
+  const int n = A.n, q = A.q, ldn = A.ldn, T = A.tpr;
+  const int R = A.res.R, r0 = min(n, lb * R), r1 = min(n, r0 + R);
+  const int L = A.res.hinfo[2 * lb], own = A.res.hinfo[2 * lb + 1], hm = A.res.hmax;
+  res::Team team{A.flags, &A.bar->err, lb, nb, A.res.cluster, 0u};
+  // the halo: FP64 x of the residual phase over rs and p (2 ES bytes an entry)
+  V *rs = reinterpret_cast<V *>(dyn), *p = rs + hm, *v = p + hm, *hat = v + hm;
+  V *d = hat + hm;                                  // own rows' correction
+  S *dinv = reinterpret_cast<S *>(d + R);
+  int *list = reinterpret_cast<int *>(dinv + hm);
+  double *xs = reinterpret_cast<double *>(dyn);
+  V *pubt = reinterpret_cast<V *>(A.pubt), *pubv = reinterpret_cast<V *>(A.pubv);
+  const S *val = reinterpret_cast<const S *>(A.valin);
+  for (int e = tid; e < L; e += RES_NT) {
+    const int c = __ldg(A.res.hlist + (size_t)lb * A.res.hstride + e);
+    list[e] = c;
+    dinv[e] = IA::ldg(reinterpret_cast<const S *>(A.dinvin) + c);
+  }
+  res::Rows<S, E, ES> row;
+  row.place(r0, r1, T);
+  row.indices(q, ldn, T, A.res.lidx);
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    const int j = row.lg + u * T;
+    row.a[u] = (row.i >= 0 && j < q) ? IA::ldg(val + (size_t)j * ldn + row.i) : IA::szero();
+  }
+  S rh[NR];
+#pragma unroll
+  for (int k = 0; k < NR; ++k) rh[k] = IA::szero();
+  if (tid < NR) {
+    IRS &c = ks[tid];
+    c.bnorm = 1.0;
+    c.relres = c.rho = c.alpha = c.omega = c.beta = c.r0 = c.snorm = 0.0;
+    c.state = KRY_RUNNING;
+    c.sweeps = c.it = c.inner_it = 0;
+    c.in_sweep = c.inner = c.half = c.zero = 0;
+  }
+  // every CTA of a cluster has started before any writes to another
+  bool ok = true;
+  if (team.cluster) res::team_barrier(team);
+  else __syncthreads();
+  const int lane = tid & 31;
+
+  // sum over the T lanes of a row, complete on its first lane
+  auto row_sum = [&](typename IA::A s) {
+    typename IA::A t = s;
+    for (int u = 1; u < T; ++u) t = IA::add(t, IA::shfl(s, (lane + u) & 31));
+    return t;
+  };
+  // (A hat) of this lane's row
+  auto spmv = [&](typename IA::A (&o)[NR]) {
+#pragma unroll
+    for (int k = 0; k < NR; ++k) o[k] = IA::zero();
+    const unsigned char *hb = reinterpret_cast<const unsigned char *>(hat);
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const V x = *reinterpret_cast<const V *>(hb + row.at(u));
+#pragma unroll
+      for (int k = 0; k < NR; ++k) IA::madd(o[k], row.a[u], x.x[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < NR; ++k) o[k] = row_sum(o[k]);
+  };
+
+  for (;;) {
+    // ---------------- R: FP64 residual, published in the inner arithmetic
+    bool part[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) part[k] = ks[k].state == KRY_RUNNING;
+    {
+      for (int e = tid; e < L; e += RES_NT) {
+        const int c = list[e];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) xs[e * NR + k] = __ldcg(A.x[k] + c);
+      }
+      __syncthreads();
+      double ax[NR];
+#pragma unroll
+      for (int k = 0; k < NR; ++k) ax[k] = 0.0;
+      if (row.i >= 0) {
+#pragma unroll 4
+        for (int j = row.lg; j < q; j += T) {
+          const size_t e = (size_t)j * ldn + row.i;
+          const double a = __ldg(A.val64 + e);
+          const double *x = xs + (int)__ldg(A.res.lidx + e) * NR;
+#pragma unroll
+          for (int k = 0; k < NR; ++k) ax[k] += a * x[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        const double s = ax[k];
+        for (int u = 1; u < T; ++u) ax[k] += __shfl_sync(0xffffffffu, s, (lane + u) & 31);
+      }
+      double acc[res::pow2_ge(2 * NR)];
+#pragma unroll
+      for (int k = 0; k < res::pow2_ge(2 * NR); ++k) acc[k] = 0.0;
+      if (row.lead) {
+        V rf;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+          const double bi = __ldg(A.b[k] + row.i), ri = bi - ax[k];
+          rf.x[k] = IA::from_double(ri);
+          if (part[k]) {
+            rh[k] = rf.x[k];
+            acc[2 * k] = bi * bi;
+            acc[2 * k + 1] = ri * ri;
+          }
+        }
+        pubt[row.i] = rf;
+      }
+      ok = res::team_totals<2 * NR>(team, acc, tot64, wsum64, cpart64,
+                                     reinterpret_cast<double *>(A.res.part));
+      if (!ok) break;
+      if (tid == 0) {
+        int any = 0;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+          IRS &c = ks[k];
+          c.in_sweep = 0;
+          c.inner = 0;
+          c.zero = 0;
+          if (part[k]) {
+            if (c.sweeps == 0) c.bnorm = sqrt(tot64[2 * k]);
+            if (c.bnorm == 0.0) {
+              c.relres = 0.0;
+              c.state = KRY_OK;
+              c.zero = 1;
+            } else {
+              const double rr = tot64[2 * k + 1];
+              c.relres = sqrt(rr) / c.bnorm;
+              if (!(c.relres == c.relres)) c.state = KRY_DIVERGED;
+              else if (c.relres <= A.tol) c.state = KRY_OK;
+              else if (c.sweeps >= A.max_sweeps || c.it >= A.maxit) c.state = KRY_NOCONV;
+              else {
+                c.in_sweep = 1;
+                c.inner = 1;
+                c.inner_it = 0;
+                c.rho = rr;
+                c.r0 = sqrt(rr);
+                lim2[k] = (A.inner_tol * c.r0) * (A.inner_tol * c.r0);
+                big2[k] = (1e3 * c.r0) * (1e3 * c.r0);
+                c.alpha = c.omega = c.beta = 0.0;
+                any = 1;
+              }
+            }
+          }
+          co.run[k] = c.inner;
+          co.alp[k] = co.omg[k] = co.nomg[k] = co.bet[k] = co.nalp[k] = IA::coef(0.0);
+        }
+        co.any = any;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < NR; ++k)
+        if (ks[k].zero) {
+          for (int i = r0 + tid; i < r1; i += RES_NT) A.x[k][i] = 0.0;
+        }
+      if (!co.any) break;
+      for (int e = tid; e < R; e += RES_NT) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) d[e].x[k] = IA::szero();
+      }
+    }
+
+    // ---------------- inner BiCGSTAB on A d = r
+    bool first = true;
+    while (co.any) {
+      // A: r = s - omega t; d += alpha p^ + omega s^; p = r + beta (p - omega v);
+      // v = A p^, partials (r^, v), (r, r)
+      bool run[NR];
+#pragma unroll
+      for (int k = 0; k < NR; ++k) run[k] = co.run[k] != 0;
+      for (int e = tid; e < L; e += RES_NT) {
+        const V t = res::ldv(pubt + list[e]);
+        const S di = dinv[e];
+        const bool mine = e >= own && e < own + (r1 - r0);
+        V h;
+        if (first) {
+          rs[e] = t;
+          p[e] = t;
+#pragma unroll
+          for (int k = 0; k < NR; ++k) h.x[k] = IA::mul(t.x[k], di);
+        } else {
+          V r = rs[e], pe = p[e];
+          const V ve = v[e];
+          if (mine) {
+            V de = d[e - own];
+#pragma unroll
+            for (int k = 0; k < NR; ++k)
+              if (run[k])
+                de.x[k] = IA::axpy(IA::axpy(de.x[k], co.alp[k], IA::mul(pe.x[k], di)), co.omg[k],
+                                   IA::mul(r.x[k], di));
+            d[e - own] = de;
+          }
+#pragma unroll
+          for (int k = 0; k < NR; ++k) {
+            r.x[k] = IA::axpy(r.x[k], co.nomg[k], t.x[k]);
+            pe.x[k] = IA::axpy(r.x[k], co.bet[k], IA::axpy(pe.x[k], co.nomg[k], ve.x[k]));
+            h.x[k] = IA::mul(pe.x[k], di);
+          }
+          rs[e] = r;
+          p[e] = pe;
+        }
+        hat[e] = h;
+      }
+      first = false;
+      __syncthreads();
+      {
+        typename IA::A av[NR];
+        spmv(av);
+        PT acc[res::pow2_ge(2 * NR)];
+#pragma unroll
+        for (int k = 0; k < res::pow2_ge(2 * NR); ++k) acc[k] = PT(0.f);
+        if (row.lead) {
+          V vn;
+          const V ri = rs[own + row.rl];
+#pragma unroll
+          for (int k = 0; k < NR; ++k) {
+            vn.x[k] = IA::from_acc(av[k]);
+            typename IA::A x = IA::zero(), y = IA::zero();
+            if (run[k]) {
+              IA::madd(x, rh[k], vn.x[k]);
+              IA::madd(y, ri.x[k], ri.x[k]);
+            }
+            acc[2 * k] = IA::part(x);
+            acc[2 * k + 1] = IA::part(y);
+          }
+          pubv[row.i] = vn;
+        }
+        ok = res::team_totals<2 * NR>(team, acc, tot, wsum, cpart,
+                                      reinterpret_cast<PT *>(A.res.part));
+      }
+      if (!ok) break;
+      if (tid < NR) {
+        IRS &c = ks[tid];
+        if (co.run[tid]) {
+          const double rr = IA::pd(tot[2 * tid + 1]);
+          // d now holds every step up to the previous iteration
+          if (!isfinite(rr) || (c.inner_it > 0 && rr <= lim2[tid]) || rr > big2[tid] ||
+              c.inner_it >= A.inner_maxit || c.it >= A.maxit) {
+            c.inner = 0;
+          } else {
+            const double al = c.rho / IA::pd(tot[2 * tid]);
+            if (!isfinite(al) || fabs(al) > 1e30) {
+              c.inner = 0;  // breakdown: keep the correction so far
+            } else {
+              c.alpha = al;
+              co.alp[tid] = IA::coef(al);
+              co.nalp[tid] = IA::coef(-al);
+            }
+          }
+          co.run[tid] = c.inner;
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {
+        int any = 0;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) any |= co.run[k];
+        co.any = any;
+      }
+#pragma unroll
+      for (int k = 0; k < NR; ++k) run[k] = co.run[k] != 0;
+      bool anyc = false;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) anyc |= run[k];
+      if (!anyc) break;
+
+      // C: s = r - alpha v, t = A s^, partials (s,s) (t,t) (t,s) (r^,s) (r^,t)
+      for (int e = tid; e < L; e += RES_NT) {
+        const V ve = res::ldv(pubv + list[e]);
+        const S di = dinv[e];
+        V s = rs[e], h;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+          s.x[k] = IA::axpy(s.x[k], co.nalp[k], ve.x[k]);
+          h.x[k] = IA::mul(s.x[k], di);
+        }
+        rs[e] = s;
+        v[e] = ve;
+        hat[e] = h;
+      }
+      __syncthreads();
+      {
+        typename IA::A at[NR];
+        spmv(at);
+        PT acc[res::pow2_ge(5 * NR)];
+#pragma unroll
+        for (int k = 0; k < res::pow2_ge(5 * NR); ++k) acc[k] = PT(0.f);
+        if (row.lead) {
+          V tn;
+          const V si = rs[own + row.rl];
+#pragma unroll
+          for (int k = 0; k < NR; ++k) {
+            tn.x[k] = IA::from_acc(at[k]);
+            if (run[k]) {
+              const S s = si.x[k], t = tn.x[k];
+              typename IA::A z[5];
+#pragma unroll
+              for (int m = 0; m < 5; ++m) z[m] = IA::zero();
+              IA::madd(z[0], s, s);
+              IA::madd(z[1], t, t);
+              IA::madd(z[2], t, s);
+              IA::madd(z[3], rh[k], s);
+              IA::madd(z[4], rh[k], t);
+#pragma unroll
+              for (int m = 0; m < 5; ++m) acc[5 * k + m] = IA::part(z[m]);
+            }
+          }
+          pubt[row.i] = tn;
+        }
+        ok = res::team_totals<5 * NR>(team, acc, tot, wsum, cpart,
+                                      reinterpret_cast<PT *>(A.res.part));
+      }
+      if (!ok) break;
+      if (tid < 32) {
+        // omega = ts / tt, rho' = (r^,s) - omega (r^,t), beta = rho' (alpha /
+        // rho) / omega: an FP64 division takes 430 cycles here, so the three
+        // run side by side on lanes 4 k .. 4 k + 2
+        const int k = lane >> 2, o = lane & 3;
+        double ss = 0.0, tt = 1.0, ts = 1.0, rhs = 0.0, rht = 0.0, num = 1.0, den = 1.0;
+        if (k < NR) {
+          ss = IA::pd(tot[5 * k + 0]);
+          tt = IA::pd(tot[5 * k + 1]);
+          ts = IA::pd(tot[5 * k + 2]);
+          rhs = IA::pd(tot[5 * k + 3]);
+          rht = IA::pd(tot[5 * k + 4]);
+          num = o == 0 ? ts : o == 1 ? tt : ks[k].alpha;
+          den = o == 0 ? tt : o == 1 ? ts : ks[k].rho;
+        }
+        const double quo = num / den;
+        const double om0 = __shfl_sync(0xffffffffu, quo, lane & ~3);
+        const double iom = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 1);
+        const double ar = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 2);
+        if (k < NR && o == 0) {
+          IRS &c = ks[k];
+          co.fin[k] = 0;
+          if (co.run[k]) {
+            c.it++;
+            c.inner_it++;
+            const double om = tt == 0.0 ? 0.0 : om0;
+            const double rho_new = rhs - om * rht;
+            const double be = (om == 0.0 || c.rho == 0.0) ? 0.0 : rho_new * ar * iom;
+            if (!isfinite(ss) || ss > big2[k] || ss <= lim2[k] || !isfinite(om) ||
+                !isfinite(be) || fabs(be) > 1e30 || om == 0.0 || rho_new == 0.0) {
+              // stop after the half step d += alpha p^ (valid whenever alpha
+              // is finite); a non-finite s drops the step altogether
+              co.fin[k] = isfinite(ss) && ss <= big2[k] ? 1 : 0;
+              c.inner = 0;
+              co.run[k] = 0;
+            } else {
+              c.rho = rho_new;
+              co.omg[k] = IA::coef(om);
+              co.nomg[k] = IA::coef(-om);
+              co.bet[k] = IA::coef(be);
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          int any = 0;
+#pragma unroll
+          for (int k2 = 0; k2 < NR; ++k2) any |= co.run[k2];
+          co.any = any;
+        }
+      }
+      __syncthreads();
+      bool fin[NR], anyfin = false;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        fin[k] = co.fin[k] != 0;
+        anyfin |= fin[k];
+      }
+      if (anyfin) {  // half step of the systems that stopped here
+        for (int e = tid; e < r1 - r0; e += RES_NT) {
+          const S di = dinv[own + e];
+#pragma unroll
+          for (int k = 0; k < NR; ++k)
+            if (fin[k])
+              d[e].x[k] = IA::axpy(d[e].x[k], co.alp[k], IA::mul(p[own + e].x[k], di));
+        }
+      }
+    }
+    if (!ok) break;
+    // ---------------- x += d (FP64)
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+      if (ks[k].in_sweep) {
+        for (int e = tid; e < r1 - r0; e += RES_NT)
+          A.x[k][r0 + e] = A.x[k][r0 + e] + IA::to_double(d[e].x[k]);
+      }
+    __syncthreads();
+    if (tid < NR && ks[tid].in_sweep) ks[tid].sweeps++;
+    ok = res::team_barrier(team);
+    if (!ok) break;
+  }
+
+  if (team.cluster) res::team_barrier(team);  // no CTA leaves while others may write to it
+  if (lb == 0 && tid < NR) {
+    A.out[tid].iters = ks[tid].it;
+    A.out[tid].restarts = ks[tid].sweeps;
+    A.out[tid].status = ok ? ks[tid].state : KRY_TIMEOUT;
+    A.out[tid].relres = ks[tid].relres;
+  }
+}
+
+template <int NR, class IA>
+const void *ir_res_fn(int E) {
+  if (E <= 6) return (const void *)k_ir_res<NR, IA, 6>;
+  if (E <= 12) return (const void *)k_ir_res<NR, IA, 12>;
+  if constexpr (sizeof(typename IA::S) == 4)
+    if (E <= 24) return (const void *)k_ir_res<NR, IA, 24>;
+  return nullptr;
+}
+
+// the kernel and its shared memory for a plan, or null: the rows' entries do
+// not fit the registers, or the halo not the shared memory
+const void *ir_res_kernel(int nr, int inner, int q, const ResPlan &p, size_t *smem) {
+  if (p.nb < 1 || p.hmax < 1 || p.hmax > p.hstride) return nullptr;
+  const int E = (q + p.T - 1) / p.T;
+  const size_t s = inner == INNER_FF ? 8 : 4;
+  if (s * nr * p.hmax > 65535) return nullptr;
+  *smem = 4 * s * nr * p.hmax + s * nr * p.R + s * p.hmax + 4 * (size_t)p.hmax + 16;
+  if (*smem > 200 * 1024) return nullptr;
+  if (inner == INNER_FF) return nr == 1 ? ir_res_fn<1, ArithFF>(E) : ir_res_fn<2, ArithFF>(E);
+  return nr == 1 ? ir_res_fn<1, ArithF32>(E) : ir_res_fn<2, ArithF32>(E);
+}
+
+}  // namespace
+
+// Runs the resident kernel when the plan and sizes allow it (*ran = true).
+static int ir_res_launch(rbffd_ctx *ctx, int nr, const MixedArgs &args, bool *ran) {
+  size_t smem = 0;
+  const void *fn = ir_res_kernel(nr, args.inner, args.q, args.res, &smem);
+  *ran = fn != nullptr;
+  if (!fn) return RBFFD_OK;
+  MixedArgs a = args;
+  a.tpr = args.res.T;
+  RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
+  if (!args.res.cluster) RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
+  return res_launch(ctx, args.res, fn, &a, smem, "k_ir_res");
+}
+
 // Batched launch: system cta_sys[b] owns the consecutive CTAs from
 // cta_first[s] and synchronises only with them.
 template <int NR, int NT, class IA>
@@ -629,6 +1116,9 @@ int krylov_ir_max_blocks(rbffd_ctx *ctx, int nr, int inner) {
 }
 
 int krylov_ir_launch(rbffd_ctx *ctx, int nr, int nblocks, const MixedArgs &args) {
+  bool ran = false;
+  RBFFD_TRY(ir_res_launch(ctx, nr, args, &ran));
+  if (ran) return RBFFD_OK;
   if (nblocks < 1 || nblocks > kdev::MAXB || nblocks > krylov_ir_max_blocks(ctx, nr, args.inner)) {
     set_error("krylov_ir_launch: %d blocks not co-resident", nblocks);
     return RBFFD_EINVAL;

@@ -174,6 +174,11 @@ int build(rbffd_problem *P, const rbffd_problem_desc *d) {
                         P->wl_rm, P->d_first_singular, P->per[0], P->per[1]));
   prof_end(ctx, 0);
   RBFFD_TRY(ops_pack(P));
+  P->res.hmax = 0;
+  int *d_hmax = P->d_first_singular + 1;
+  if (P->res.nb > 0)
+    RBFFD_TRY(res_halo_build(ctx, P->res, P->n, P->q, P->ldn, P->col, P->res_hlist, P->res_hinfo,
+                             P->res_lidx, d_hmax));
   P->precond = d->precond;
   // the multigrid hierarchy's host part runs on a thread of its own from
   // here; the first p' solve (amg_ready) waits for it and uploads it, so
@@ -207,9 +212,12 @@ int build(rbffd_problem *P, const rbffd_problem_desc *d) {
                                                    P->p, P->un, P->vn, P->unm1, P->vnm1, P->pc,
                                                    P->ut, P->vt);
   RBFFD_TRY(after_launch(ctx, "k_init_state"));
-  int hfs = big;
-  RBFFD_CK(cudaMemcpyAsync(&hfs, P->d_first_singular, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int back[2] = {big, 0};  // first singular cloud, longest halo list
+  RBFFD_CK(cudaMemcpyAsync(back, P->d_first_singular, (P->res.nb > 0 ? 2 : 1) * sizeof(int),
+                           cudaMemcpyDeviceToHost, st));
   RBFFD_CK(cudaStreamSynchronize(st));
+  const int hfs = back[0];
+  P->res.hmax = back[1];
   if (ctx->prof) {
     const double N = P->q + (P->degree + 1) * (P->degree + 2) / 2;
     const double flops = 2.0 * N * N * N / 3.0 + 6.0 * N * N + 10.0 * P->q * P->q;
@@ -260,14 +268,15 @@ int rbffd::amg_ready(rbffd_problem *P) {
 
 namespace {
 
-// Issue one outer iteration (no host synchronisation beyond the first p'
-// solve's wait for a hierarchy still being built).
-// The momentum solves run in the problem's precision: FP64 BiCGSTAB, or
-// (mixed) FP32 / float-float BiCGSTAB inside FP64 refinement.  The p'
-// solve follows its preconditioner: with Jacobi it takes the same
-// precision; multigrid BiCGSTAB is FP64 throughout; flexible GMRES runs its
-// Arnoldi process in FP32 inside FP64 restarts (fgmres.cu).  Every solve
-// stops on the same FP64 relative residual.
+// The resident solve of a mixed-precision system: team, lists and scratch.
+void resident_args(rbffd_problem *P, MixedArgs *m) {
+  m->res = P->res;
+  // published vectors, up to two right-hand sides side by side: r and rh,
+  // p0 and p1 of the first system are adjacent in the allocation
+  m->pubt = P->mv[0].r;
+  m->pubv = P->mv[0].p0;
+}
+
 // Issue the pressure-correction solve M x = b with the problem's p' solver
 // (no host synchronisation): flexible GMRES with the FP32 hierarchy,
 // mixed-precision Jacobi BiCGSTAB, or FP64 BiCGSTAB with the FP64
@@ -325,6 +334,7 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
     m.b[0] = b;
     m.x[0] = x;
     m.w[0] = P->mv[0];
+    resident_args(P, &m);
     m.out = P->kout + 2;
     m.tpr = krylov_threads_per_row(P->n, 1, P->kblocks1);
     return krylov_ir_launch(ctx, 1, P->kblocks1, m);
@@ -352,6 +362,14 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
   return krylov_launch(ctx, 1, P->kblocks1, a);
 }
 
+// Issue one outer iteration (no host synchronisation beyond the first p'
+// solve's wait for a hierarchy still being built).
+// The momentum solves run in the problem's precision: FP64 BiCGSTAB, or
+// (mixed) FP32 / float-float BiCGSTAB inside FP64 refinement.  The p'
+// solve follows its preconditioner: with Jacobi it takes the same
+// precision; multigrid BiCGSTAB is FP64 throughout; flexible GMRES runs its
+// Arnoldi process in FP32 inside FP64 restarts (fgmres.cu).  Every solve
+// stops on the same FP64 relative residual.
 int issue_outer(rbffd_problem *P, const rbffd_step_params *sp) {
   rbffd_ctx *ctx = P->ctx;
   prof_begin(ctx, 2);
@@ -402,6 +420,7 @@ int issue_outer(rbffd_problem *P, const rbffd_step_params *sp) {
     m.x[1] = P->vt;
     m.w[0] = P->mv[0];
     m.w[1] = P->mv[1];
+    resident_args(P, &m);
     m.out = P->kout;
     m.tpr = krylov_threads_per_row(P->n, 2, P->kblocks2);
     if (!P->has_sym) {
@@ -602,6 +621,7 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       if (P->kblocks2 > c2) P->kblocks2 = c2;
     }
     P->rblocks = ops_reduce_blocks(ctx, n);
+    P->res = res_plan(ctx, n);
     // partials: room for two right-hand sides over the larger grid (a batched
     // launch may give one member two single-RHS systems, or one system twice
     // the CTAs)
@@ -626,7 +646,7 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
     size_t o_bar = c.take<GridBarrier>(1);
     size_t o_flags = c.take<unsigned int>(256);
     size_t o_rec = c.take<Readback>(1);
-    size_t o_fs = c.take<int>(1);
+    size_t o_fs = c.take<int>(2);
     size_t o_knn = c.take<char>(P->knn_lay.bytes);
     size_t o_p32 = 0, o_a32 = 0, o_pd32 = 0, o_md32 = 0, o_mv[18] = {}, o_part64 = 0, o_part32 = 0;
     size_t o_a32b = 0, o_md32b = 0;
@@ -642,6 +662,14 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       o_part64 = c.take<double>(krylov_ir_partials64(2, kb));
       o_part32 = c.take<char>(krylov_ir_partials_inner_bytes(2, kb, P->inner));
     }
+    size_t o_hl = 0, o_hi = 0, o_li = 0, o_rp = 0;
+    if (!mixed && d->precond != RBFFD_PRECOND_AMG_FGMRES) P->res.nb = 0;
+    if (P->res.nb > 0) {
+      o_hl = c.take<int32_t>((size_t)P->res.nb * P->res.hstride);
+      o_hi = c.take<int32_t>(2 * (size_t)P->res.nb);
+      o_li = c.take<uint16_t>(lq);
+      o_rp = c.take<char>(RES_PART_BYTES);
+    }
     P->bytes = c.off;
     int rc = dev_alloc(ctx, &P->mem, P->bytes);
     if (rc != RBFFD_OK) {
@@ -650,6 +678,12 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       return rc;
     }
     char *b = (char *)P->mem;
+    if (P->res.nb > 0) {
+      P->res.hlist = P->res_hlist = (int32_t *)(b + o_hl);
+      P->res.hinfo = P->res_hinfo = (int32_t *)(b + o_hi);
+      P->res.lidx = P->res_lidx = (uint16_t *)(b + o_li);
+      P->res.part = b + o_rp;
+    }
     P->x = (double *)(b + o_x);
     P->y = (double *)(b + o_y);
     P->nx = (double *)(b + o_nx);

@@ -5,6 +5,7 @@
 #include "amg_job.cuh"
 #include "knn.cuh"
 #include "krylov.cuh"
+#include "resident.cuh"
 
 // Outer-iteration record read back by the host once per outer iteration.
 struct IterRecord {
@@ -47,6 +48,11 @@ struct rbffd_problem {
   rbffd::MixedVecs mv[2] = {};
   double *part64 = nullptr;
   void *partin = nullptr;
+  // team and halo lists of the resident solves (nb = 0: none); its arrays
+  // are in this allocation, rebuilt with the clouds
+  rbffd::ResPlan res;
+  int32_t *res_hlist = nullptr, *res_hinfo = nullptr;
+  uint16_t *res_lidx = nullptr;
   // fields
   double *u, *v, *p, *p2, *un, *vn, *unm1, *vnm1, *ut, *vt, *pc, *bu, *bv, *bp;
   // compatible p' of a pinned problem (no outlet): z = M^{-1} e_I, solved

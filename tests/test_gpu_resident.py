@@ -1,0 +1,52 @@
+"""The resident Krylov kernels (matrix in registers, halo lists in shared
+memory) against the oracle, at the sizes where their layout can go wrong:
+one CTA, one cluster and its largest size, the smallest grid team, the last
+CTA empty, every lanes-per-row and entries-per-lane class, symmetry lines
+(single right-hand sides), and a random point order, whose halo lists are
+longest.  One outer iteration to the tolerance the other parity tests use."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import ctx, rel_l2
+from paper_2106_07616_gb300 import clouds, rbffd
+
+pytestmark = pytest.mark.gpu
+FIELDS = ("u", "v", "p")
+
+
+def shuffled(fp, seed):
+    o = np.random.Generator(np.random.PCG64(seed)).permutation(fp.n)
+    for k in ("x", "y", "tag", "nx", "ny", "ubc", "vbc"):
+        setattr(fp, k, np.ascontiguousarray(getattr(fp, k)[o]))
+    if fp.pin >= 0:
+        fp.pin = int(np.nonzero(o == fp.pin)[0][0])
+    return fp
+
+
+CASES = {
+    "one_cta": lambda: clouds.kovasznay(11, dt=0.4),                       # 121 rows
+    "two_ctas": lambda: clouds.kovasznay(12, dt=0.4),                      # 144 rows
+    "cluster_q42": lambda: clouds.kovasznay(40, degree=5, q=42, dt=0.2),   # 1600 rows
+    "cluster_full": lambda: clouds.kovasznay(64, degree=2, q=12, dt=0.2),  # 4096 rows
+    "grid_least": lambda: clouds.kovasznay(65, dt=0.2),                    # 4225 rows
+    "grid_q30": lambda: clouds.cavity(90, degree=4, q=30, re=100.0),
+    "grid_shuffled": lambda: shuffled(clouds.kovasznay(66, dt=0.2), 3),
+    "symmetry": lambda: clouds.channel(61, 31, symmetry=True),
+    "last_cta_empty": lambda: clouds.channel(166, 120, dt=0.02),           # 19 920 rows
+}
+
+
+@pytest.mark.parametrize("precision", [rbffd.PREC_MIXED, rbffd.PREC_MIXED_FF])
+@pytest.mark.parametrize("case", sorted(CASES))
+def test_resident_iteration_matches_oracle(case, precision):
+    fp = CASES[case]()
+    P = rbffd.Problem(ctx(), fp, precision, precond=rbffd.PRECOND_AMG)
+    O = oracle.Problem(fp, krylov_tol=1e-12, krylov_maxit=100000)
+    dg, sg = P.simple_iterate(fp.dt, krylov_tol=1e-12, krylov_maxit=100000)
+    do, so = O.simple_iterate(fp.dt)
+    assert max(sg["relres"]) <= 1e-12
+    assert abs(dg - do) <= 1e-8 * abs(do), (dg, do)
+    for k in FIELDS:
+        assert rel_l2(P.get(k), O.get(k)) <= 1e-8, k
+    P.close()
