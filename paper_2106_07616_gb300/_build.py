@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "librbffd.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 
 SOURCES = ["context.cu", "knn.cu", "weights.cu", "krylov.cu", "krylov_mixed.cu", "resident.cu", "ops.cu", "amg.cu",
-           "amg_setup.cu", "fgmres.cu",
+           "amg_setup.cu", "fgmres.cu", "fgmres_res.cu",
            "problem.cu", "batch.cu", "server.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE,

@@ -45,4 +45,15 @@ int fgmres_batch_max_ctas(rbffd_ctx *ctx);
 int fgmres_batch_launch(rbffd_ctx *ctx, int nctas, const FgmresArgs *d_sys,
                         const int *d_cta_sys, const int *d_cta_first);
 
+// The same solve on a resident team (fgmres_res.cu), when the plan, the
+// hierarchy and the sizes allow it (*ran).  omega: level 0's smoothing
+// weight; B: the dense coarse operator, or null.
+constexpr int RES_DENSE_N = 2048;  // most level-1 rows of a dense coarse operator
+int fgmres_res_launch(rbffd_ctx *ctx, const FgmresArgs &args, const ResPlan &res,
+                      const AmgDevF &h, double omega, const float *B, bool *ran);
+// Leading dimension of the hierarchy's dense coarse operator (0: none), and
+// the operator itself, n1 x ld values.
+int fgmres_dense_ld(const AmgDevF &h);
+int fgmres_dense_build(rbffd_ctx *ctx, const AmgDevF &h, float *B);
+
 }  // namespace rbffd

@@ -85,6 +85,9 @@ void free_amg(rbffd_problem *P) {
   P->fg_mem = nullptr;
   P->fg_bytes = 0;
   P->fgV = P->fgZ = nullptr;
+  if (P->fgB) dev_free(P->ctx, P->fgB, P->fgB_bytes);
+  P->fgB = nullptr;
+  P->fgB_bytes = 0;
   P->fgR = nullptr;
   P->fgpart = nullptr;
   P->amgf = nullptr;
@@ -309,6 +312,18 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
     f.maxit = maxit;
     f.amg = P->amgf;
     f.reorth = ctx->fgmres_reorth;
+    // the resident solve's dense coarse operator, made at its first solve
+    // (batched members never need it); without memory for it the solve runs
+    // the composed cycle's phases
+    const int ld = P->res.nb > 0 && !P->fgB ? fgmres_dense_ld(P->amgf_host) : 0;
+    const size_t bytes = sizeof(float) * (size_t)ld * (ld > 0 ? P->amgf_host.lev[1].n : 0);
+    if (ld > 0 && dev_alloc(ctx, (void **)&P->fgB, bytes) == RBFFD_OK) {
+      P->fgB_bytes = bytes;
+      RBFFD_TRY(fgmres_dense_build(ctx, P->amgf_host, P->fgB));
+    }
+    bool ran = false;
+    RBFFD_TRY(fgmres_res_launch(ctx, f, P->res, P->amgf_host, P->amg_info.omega[0], P->fgB, &ran));
+    if (ran) return RBFFD_OK;
     return fgmres_launch(ctx, P->fg_blocks, f);
   }
   if (mixed && !P->amg && !jacobi) {
@@ -776,7 +791,7 @@ extern "C" void rbffd_problem_destroy(rbffd_problem *P) {
 }
 
 extern "C" size_t rbffd_problem_bytes(const rbffd_problem *P) {
-  return P ? P->bytes + P->amg_bytes + P->amg0_bytes + P->fg_bytes : 0;
+  return P ? P->bytes + P->amg_bytes + P->amg0_bytes + P->fg_bytes + P->fgB_bytes : 0;
 }
 
 static void report_levels(const AmgInfo &I, bool have_any, int32_t *levels, int32_t *rows,

@@ -109,6 +109,8 @@ struct rbffd_problem {
   float *fgV = nullptr, *fgZ = nullptr;       // FP32 basis and directions
   void *fgpart = nullptr;
   int fg_m = 0, fg_blocks = 0;
+  float *fgB = nullptr;  // dense coarse operator (fgmres_res.cu), or null
+  size_t fgB_bytes = 0;
 };
 
 namespace rbffd {
