@@ -35,6 +35,7 @@ namespace {
 
 constexpr int LDH = FG_MAXM + 1;
 constexpr int MAXV = FG_MAXM + 1;   // vectors V of a restart that are kept
+constexpr int MAXR1 = 256;          // level-1 rows a CTA may own
 
 struct FgResArgs {
   FgmresArgs f;
@@ -57,6 +58,7 @@ struct FgResArgs {
 
 struct FgState {
   double bnorm, beta, scale, relres;
+  float gtol;  // |g_{j+1}| at which the restart's residual estimate meets the tolerance
   int it, restarts, state, k, stop;
 };
 
@@ -106,7 +108,8 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
   __shared__ float tot[32], cpart[2 * 32 * RES_CLUSTER];
   __shared__ double tot64[2], wsum64[2 * 32], cpart64[2 * 2 * RES_CLUSTER];
   __shared__ FgState st;
-  __shared__ float rowpart[64];
+  __shared__ float rowpart[32];
+  __shared__ int rptr[MAXR1 + 1];
   extern __shared__ __align__(16) unsigned char dyn[];
   const FgmresArgs &F = A.f;
   const int lb = blockIdx.x, nb = gridDim.x, tid = threadIdx.x;
@@ -146,6 +149,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
   // this CTA's rows of R~ and P~: contiguous entries of the CSR arrays
   const int rs0 = k1 > k0 ? __ldg(A.R0.ptr + k0) : 0, rs1 = k1 > k0 ? __ldg(A.R0.ptr + k1) : 0;
   const int ps0 = nr > 0 ? __ldg(A.P0.ptr + r0) : 0, ps1 = nr > 0 ? __ldg(A.P0.ptr + r1) : 0;
+  for (int k = tid; k <= k1 - k0; k += RES_NT) rptr[k] = __ldg(A.R0.ptr + k0 + k) - rs0;
   const bool rres = rs1 - rs0 <= A.rcap, pres = ps1 - ps0 <= A.pcap;
   if (rres)
     for (int e = tid; e < rs1 - rs0; e += RES_NT)
@@ -159,10 +163,8 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
     pe = __ldg(A.P0.ptr + row.i + 1);
   }
   if (A.B && A.bres)
-    for (int e = tid; e < (k1 - k0) * n1; e += RES_NT) {
-      const int i = e / n1, c = e - i * n1;
-      Bs[i * A.ldb + c] = __ldg(A.B + (size_t)(k0 + i) * A.ldb + c);
-    }
+    for (int e = tid; e < (k1 - k0) * A.ldb; e += RES_NT)
+      Bs[e] = __ldg(A.B + (size_t)k0 * A.ldb + e);
   if (tid == 0) {
     st.bnorm = st.beta = 0.0;
     st.relres = 1.0;
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
         A.u[r0 + r] = v;
       }
       if (tid == 0) {
+        st.gtol = (float)(F.tol * st.bnorm / st.beta);
         g[0] = 1.0f;
         for (int k = 1; k <= FG_MAXM; ++k) g[k] = 0.0f;
         st.k = 0;
@@ -304,17 +307,17 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
         // R~'s gathers are in flight with the halo's
         for (int task = warp; task < (k1 - k0) * nparts; task += 32) {
           const int k = task / nparts, part = task - k * nparts;
-          const int s = __ldg(A.R0.ptr + k0 + k), e1 = __ldg(A.R0.ptr + k0 + k + 1);
+          const int s = rptr[k], e1 = rptr[k + 1];
           float t = 0.0f;
           if (rres) {
 #pragma unroll 4
             for (int e = s + lane + 32 * part; e < e1; e += 32 * nparts) {
-              const int2 ce = Rs[e - rs0];
+              const int2 ce = Rs[e];
               t = fmaf(__int_as_float(ce.y), __ldcg(A.u + ce.x), t);
             }
           } else {
 #pragma unroll 4
-            for (int e = s + lane + 32 * part; e < e1; e += 32 * nparts)
+            for (int e = rs0 + s + lane + 32 * part; e < rs0 + e1; e += 32 * nparts)
               t = fmaf(__ldg(A.R0.val + e), __ldcg(A.u + __ldg(A.R0.col + e)), t);
           }
           t = res::warp_total(t);
@@ -345,14 +348,27 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
       if (!res::team_barrier(team)) { ok = false; break; }
       // ---- B: y_1
       if (A.B) {
-        for (int e = tid; e < n1; e += RES_NT) c1[e] = __ldcg(A.b1 + e);
+        for (int e = tid; e < max(n1, A.ldb); e += RES_NT)
+          c1[e] = e < n1 ? __ldcg(A.b1 + e) : 0.0f;
         __syncthreads();
         for (int task = warp; task < (k1 - k0) * nparts; task += 32) {
           const int k = task / nparts, part = task - k * nparts;
           const float *b = A.bres ? Bs + k * A.ldb : A.B + (size_t)(k0 + k) * A.ldb;
           float t = 0.0f;
-#pragma unroll 8
-          for (int e = lane + 32 * part; e < n1; e += 32 * nparts) t = fmaf(b[e], c1[e], t);
+          if ((A.ldb & 3) == 0) {  // rows and b_1 padded to whole quadruples
+            const float4 *b4 = reinterpret_cast<const float4 *>(b);
+            const float4 *c4 = reinterpret_cast<const float4 *>(c1);
+#pragma unroll 4
+            for (int e = lane + 32 * part; e < A.ldb / 4; e += 32 * nparts) {
+              const float4 x = b4[e], y = c4[e];
+              t = fmaf(x.x, y.x, t);
+              t = fmaf(x.y, y.y, t);
+              t = fmaf(x.z, y.z, t);
+              t = fmaf(x.w, y.w, t);
+            }
+          } else {
+            for (int e = lane + 32 * part; e < n1; e += 32 * nparts) t = fmaf(b[e], c1[e], t);
+          }
           t = res::warp_total(t);
           if (lane == 0) {
             if (nparts == 1) A.y1[k0 + k] = t;
@@ -487,8 +503,8 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
           g[j] = cs[j] * g[j];
           st.it++;
           st.k = j + 1;
-          const double est = fabs((double)g[j + 1]) * st.beta / st.bnorm;
-          st.stop = !(est == est) ? 2 : (est <= F.tol || hn == 0.0f || st.it >= F.maxit) ? 1 : 0;
+          const float ga = fabsf(g[j + 1]);
+          st.stop = !(ga == ga) ? 2 : (ga <= st.gtol || hn == 0.0f || st.it >= F.maxit) ? 1 : 0;
           if (st.stop == 2) st.state = KRY_DIVERGED;
         }
       }
@@ -573,11 +589,11 @@ bool fg_layout(FgResArgs &a, size_t *smem) {
   a.o_w = take(4 * (size_t)hm);
   a.o_work = take(8 * (size_t)hm);
   const size_t coarse = a.B ? 0 : (size_t)(a.C.nc + R1);
-  a.o_c1 = take(4 * (coarse > (size_t)n1 ? coarse : (size_t)n1));
+  a.o_c1 = take(4 * (coarse > (size_t)n1 ? coarse : (size_t)n1) + 16);
   a.ldv = R;
   while (a.ldv % 32 != (32 / a.res.T) % 32) ++a.ldv;
   const size_t vec = 4 * (size_t)a.ldv;
-  if (at + vec > limit) return false;
+  if (at + vec > limit || R1 > MAXR1) return false;
   size_t left = limit - at - round16(vec);  // the vector w always has a place
   // basis vectors first, then B, then the transfer slabs: B and the slabs are
   // read once a step, a basis vector four times

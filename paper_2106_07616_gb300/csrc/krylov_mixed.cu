@@ -595,11 +595,31 @@ __global__ void __launch_bounds__(NT) k_bicgstab_ir(MixedArgs A) {
 // 20.2 -> 11.6 ms, Kovasznay 50^2 (one cluster) 6.9 -> 4.9 ms.
 namespace {
 
+// What every thread of the CTA needs of the recurrences' scalars, and the
+// scalars themselves.  rho, alpha and omega are float-float: an FP64
+// division takes over 400 cycles on GB300 and the chain of them took 1.4 us
+// after phase A and 3 us after phase C, of 11 us an iteration; a float-float
+// division (two FP32 quotients and an exact remainder) keeps 46 bits of
+// sums that have 24 (or 48), and the coefficients are rounded to the inner
+// arithmetic right after.
 template <int NR, class IA>
 struct IrCoef {
   typename IA::C alp[NR], omg[NR], nomg[NR], bet[NR], nalp[NR];
   int run[NR], fin[NR], any;
+  ff rho[NR], alpha[NR];
+  float lim2[NR], big2[NR];  // (inner_tol r0)^2, (1e3 r0)^2 of the sweep
+  int it[NR], inner_it[NR];
 };
+
+__device__ __forceinline__ ff ff_of(float v) { return ff(v, 0.f); }
+__device__ __forceinline__ ff ff_of(ff v) { return v; }
+__device__ __forceinline__ void coef_of(ff v, float &o) { o = v.hi; }
+__device__ __forceinline__ void coef_of(ff v, ff &o) { o = v; }
+__device__ __forceinline__ ff ff_div(ff a, ff b) {
+  const float q = __fdiv_rn(a.hi, b.hi);
+  const ff r = ff_add(a, ff_neg(ff_mul(b, ff(q, 0.f))));
+  return ff_fast_two_sum(q, __fdiv_rn(r.hi, b.hi));
+}
 
 template <int NR, class IA, int E>
 __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
@@ -613,7 +633,6 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
   __shared__ PT tot[5 * NR];
   __shared__ double tot64[2 * NR];
   __shared__ IRS ks[NR];
-  __shared__ double lim2[NR], big2[NR];  // (inner_tol r0)^2, (1e3 r0)^2 of the sweep
   __shared__ IrCoef<NR, IA> co;
   extern __shared__ __align__(16) unsigned char dyn[];
   const int lb = blockIdx.x, nb = gridDim.x, tid = threadIdx.x;
@@ -753,17 +772,16 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
               else {
                 c.in_sweep = 1;
                 c.inner = 1;
-                c.inner_it = 0;
-                c.rho = rr;
-                c.r0 = sqrt(rr);
-                lim2[k] = (A.inner_tol * c.r0) * (A.inner_tol * c.r0);
-                big2[k] = (1e3 * c.r0) * (1e3 * c.r0);
-                c.alpha = c.omega = c.beta = 0.0;
+                co.rho[k] = ff_from_double(rr);
+                co.lim2[k] = (float)(A.inner_tol * A.inner_tol * rr);
+                co.big2[k] = (float)(1e6 * rr);
                 any = 1;
               }
             }
           }
           co.run[k] = c.inner;
+          co.it[k] = c.it;
+          co.inner_it[k] = 0;
           co.alp[k] = co.omg[k] = co.nomg[k] = co.bet[k] = co.nalp[k] = IA::coef(0.0);
         }
         co.any = any;
@@ -850,25 +868,21 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
                                       reinterpret_cast<PT *>(A.res.part));
       }
       if (!ok) break;
-      if (tid < NR) {
-        IRS &c = ks[tid];
-        if (co.run[tid]) {
-          const double rr = IA::pd(tot[2 * tid + 1]);
-          // d now holds every step up to the previous iteration
-          if (!isfinite(rr) || (c.inner_it > 0 && rr <= lim2[tid]) || rr > big2[tid] ||
-              c.inner_it >= A.inner_maxit || c.it >= A.maxit) {
-            c.inner = 0;
+      if (tid < NR && co.run[tid]) {
+        const float rr = ff_of(tot[2 * tid + 1]).hi;
+        // d now holds every step up to the previous iteration
+        if (!isfinite(rr) || (co.inner_it[tid] > 0 && rr <= co.lim2[tid]) ||
+            rr > co.big2[tid] || co.inner_it[tid] >= A.inner_maxit || co.it[tid] >= A.maxit) {
+          co.run[tid] = 0;
+        } else {
+          const ff al = ff_div(co.rho[tid], ff_of(tot[2 * tid]));
+          if (!isfinite(al.hi) || fabsf(al.hi) > 1e30f) {
+            co.run[tid] = 0;  // breakdown: keep the correction so far
           } else {
-            const double al = c.rho / IA::pd(tot[2 * tid]);
-            if (!isfinite(al) || fabs(al) > 1e30) {
-              c.inner = 0;  // breakdown: keep the correction so far
-            } else {
-              c.alpha = al;
-              co.alp[tid] = IA::coef(al);
-              co.nalp[tid] = IA::coef(-al);
-            }
+            co.alpha[tid] = al;
+            coef_of(al, co.alp[tid]);
+            coef_of(ff_neg(al), co.nalp[tid]);
           }
-          co.run[tid] = c.inner;
         }
       }
       __syncthreads();
@@ -933,45 +947,33 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
       }
       if (!ok) break;
       if (tid < 32) {
-        // omega = ts / tt, rho' = (r^,s) - omega (r^,t), beta = rho' (alpha /
-        // rho) / omega: an FP64 division takes 430 cycles here, so the three
-        // run side by side on lanes 4 k .. 4 k + 2
-        const int k = lane >> 2, o = lane & 3;
-        double ss = 0.0, tt = 1.0, ts = 1.0, rhs = 0.0, rht = 0.0, num = 1.0, den = 1.0;
-        if (k < NR) {
-          ss = IA::pd(tot[5 * k + 0]);
-          tt = IA::pd(tot[5 * k + 1]);
-          ts = IA::pd(tot[5 * k + 2]);
-          rhs = IA::pd(tot[5 * k + 3]);
-          rht = IA::pd(tot[5 * k + 4]);
-          num = o == 0 ? ts : o == 1 ? tt : ks[k].alpha;
-          den = o == 0 ? tt : o == 1 ? ts : ks[k].rho;
-        }
-        const double quo = num / den;
-        const double om0 = __shfl_sync(0xffffffffu, quo, lane & ~3);
-        const double iom = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 1);
-        const double ar = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 2);
-        if (k < NR && o == 0) {
-          IRS &c = ks[k];
+        if (lane < NR) {
+          const int k = lane;
           co.fin[k] = 0;
           if (co.run[k]) {
-            c.it++;
-            c.inner_it++;
-            const double om = tt == 0.0 ? 0.0 : om0;
-            const double rho_new = rhs - om * rht;
-            const double be = (om == 0.0 || c.rho == 0.0) ? 0.0 : rho_new * ar * iom;
-            if (!isfinite(ss) || ss > big2[k] || ss <= lim2[k] || !isfinite(om) ||
-                !isfinite(be) || fabs(be) > 1e30 || om == 0.0 || rho_new == 0.0) {
+            const ff tt = ff_of(tot[5 * k + 1]), ts = ff_of(tot[5 * k + 2]);
+            const float ss = ff_of(tot[5 * k]).hi;
+            co.it[k]++;
+            co.inner_it[k]++;
+            // omega = ts / tt, rho' = (r^,s) - omega (r^,t),
+            // beta = (rho' / rho) (alpha / omega)
+            const ff om = tt.hi == 0.f ? ff(0.f) : ff_div(ts, tt);
+            const ff rho_new =
+                ff_add(ff_of(tot[5 * k + 3]), ff_neg(ff_mul(om, ff_of(tot[5 * k + 4]))));
+            const ff be = (om.hi == 0.f || co.rho[k].hi == 0.f)
+                              ? ff(0.f)
+                              : ff_mul(ff_div(rho_new, co.rho[k]), ff_div(co.alpha[k], om));
+            if (!isfinite(ss) || ss > co.big2[k] || ss <= co.lim2[k] || !isfinite(om.hi) ||
+                !isfinite(be.hi) || fabsf(be.hi) > 1e30f || om.hi == 0.f || rho_new.hi == 0.f) {
               // stop after the half step d += alpha p^ (valid whenever alpha
               // is finite); a non-finite s drops the step altogether
-              co.fin[k] = isfinite(ss) && ss <= big2[k] ? 1 : 0;
-              c.inner = 0;
+              co.fin[k] = isfinite(ss) && ss <= co.big2[k] ? 1 : 0;
               co.run[k] = 0;
             } else {
-              c.rho = rho_new;
-              co.omg[k] = IA::coef(om);
-              co.nomg[k] = IA::coef(-om);
-              co.bet[k] = IA::coef(be);
+              co.rho[k] = rho_new;
+              coef_of(om, co.omg[k]);
+              coef_of(ff_neg(om), co.nomg[k]);
+              coef_of(be, co.bet[k]);
             }
           }
         }
@@ -1010,7 +1012,10 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           A.x[k][r0 + e] = A.x[k][r0 + e] + IA::to_double(d[e].x[k]);
       }
     __syncthreads();
-    if (tid < NR && ks[tid].in_sweep) ks[tid].sweeps++;
+    if (tid < NR && ks[tid].in_sweep) {
+      ks[tid].sweeps++;
+      ks[tid].it = co.it[tid];
+    }
     ok = res::team_barrier(team);
     if (!ok) break;
   }
