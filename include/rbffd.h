@@ -550,6 +550,18 @@ int rbffd_plan_work_lists(int32_t m, const double *work, const int32_t *cap, con
                           int32_t cmax, double scale, int32_t *nctas, int32_t *team_size,
                           int32_t *nteams, int32_t *member_team);
 
+/* The plan the batched launches use (host only): as rbffd_plan_work_lists,
+ * but the teams differ in size, chosen so that the team that finishes last
+ * finishes soonest, a solve of rows r and work w on c CTAs taking
+ * (w / r) (512 + r / c).  Solve i goes to team member_team[i] of
+ * member_ctas[i] CTAs (at most cap[i], and what 8 threads a row fill);
+ * *nctas = the CTAs of all teams, at most cmax; *span = the longest team's
+ * time (both nullable).  The autotuner's candidates other than scale 1 use
+ * the equal teams of rbffd_plan_work_lists.  Errors: RBFFD_EINVAL. */
+int rbffd_plan_teams(int32_t m, const double *work, const int32_t *cap, const int32_t *rows,
+                     int32_t cmax, int32_t *member_team, int32_t *member_ctas, int32_t *nctas,
+                     double *span);
+
 /* -------------------------------------------------------------- serving */
 
 /* A request server with continuous batching (the serving workload; the

@@ -189,6 +189,110 @@ static TeamPlan plan_teams(const std::vector<double> &work, const std::vector<in
   return T;
 }
 
+// Fixed cost of a Krylov iteration in rows: its exchanges and dependent L2
+// round trips take as long as the arithmetic of about this many rows of one
+// CTA (multigrid BiCGSTAB: 60 us an iteration on a problem too small to
+// matter, against 80 ns a row and CTA; momentum with two right-hand sides:
+// 28 us against 60 ns).
+constexpr double PLAN_LATENCY_ROWS = 512.0;
+
+// A work list whose teams may differ in size: the systems form ngroups
+// groups (LPT on their work), every group one team, and the CTAs go one by
+// one to the team that would finish last,
+//   time(team) = sum over its systems of iterations (latency + rows / CTAs),
+// as far as its systems' partial sums (cap) and 8 threads a row allow.  The
+// number of groups with the least longest time is taken; with as many groups
+// as systems everything runs at once.  *span: that time.
+static TeamPlan plan_groups(const std::vector<double> &work, const std::vector<int> &cap,
+                            const std::vector<int> &rows, int cmax, int ngroups, double *span) {
+  const int m = (int)work.size();
+  std::vector<int> order(m);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return work[a] > work[b]; });
+  struct Group {
+    double its = 0.0, work = 0.0;  // iterations (fixed cost), rows x iterations
+    int cap = kdev::MAXB, ctas = 1;
+    std::vector<int> list;
+    double time(int c) const { return its * PLAN_LATENCY_ROWS + work / c; }
+  };
+  std::vector<Group> G(ngroups);
+  for (int i : order) {
+    Group *best = &G[0];
+    for (Group &g : G)
+      if (g.work < best->work) best = &g;
+    best->work += work[i];
+    best->its += work[i] / rows[i];
+    const int rowcap = std::max(1, (int)((rows[i] * 8LL + KB_NT - 1) / KB_NT));
+    best->cap = std::min({best->cap, cap[i], std::max(rowcap, 1)});
+    best->list.push_back(i);
+  }
+  auto slower = [&](int a, int b) { return G[a].time(G[a].ctas) < G[b].time(G[b].ctas); };
+  std::vector<int> heap(ngroups);
+  std::iota(heap.begin(), heap.end(), 0);
+  std::make_heap(heap.begin(), heap.end(), slower);
+  *span = 0.0;
+  int left = cmax - ngroups;
+  while (!heap.empty()) {
+    std::pop_heap(heap.begin(), heap.end(), slower);
+    Group &g = G[heap.back()];
+    if (left > 0 && g.ctas < g.cap) {
+      ++g.ctas;
+      --left;
+      std::push_heap(heap.begin(), heap.end(), slower);
+    } else {
+      *span = std::max(*span, g.time(g.ctas));
+      heap.pop_back();  // at its largest, or no CTA left: the time is final
+    }
+  }
+  TeamPlan T;
+  T.info_and_list.assign(4 * ngroups, 0);
+  T.nb.assign(m, 1);
+  for (int t = 0; t < ngroups; ++t) {
+    T.info_and_list[4 * t] = T.nctas;
+    T.info_and_list[4 * t + 1] = G[t].ctas;
+    T.info_and_list[4 * t + 2] = (int)T.info_and_list.size();
+    for (int i : G[t].list) {
+      T.nb[i] = G[t].ctas;
+      T.info_and_list.push_back(i);
+    }
+    T.info_and_list[4 * t + 3] = (int)T.info_and_list.size();
+    T.nctas += G[t].ctas;
+    T.cta_team.resize(T.nctas, t);
+  }
+  return T;
+}
+
+static TeamPlan plan_by_time(const std::vector<double> &work, const std::vector<int> &cap,
+                             const std::vector<int> &rows, int cmax, double *span) {
+  const int m = (int)work.size(), gmax = std::min(m, cmax);
+  TeamPlan best;
+  *span = 1e300;
+  // every group count up to 16, then in steps of a sixteenth
+  for (int g = 1; g <= gmax; g = g < gmax ? std::min(gmax, g + std::max(1, g / 16)) : gmax + 1) {
+    double s = 0.0;
+    TeamPlan T = plan_groups(work, cap, rows, cmax, g, &s);
+    if (s < *span) {
+      *span = s;
+      best = std::move(T);
+    }
+  }
+  return best;
+}
+
+// The plan a launch takes: by time, or, for the autotuner's other scales, the
+// equal teams of plan_teams.  Why: equal teams are as small as the smallest
+// member's partial sums allow (23 CTAs for 1 444 rows), and members beyond
+// the teams wait for their turn; 16 members of 1 444 to 50 625 rows took
+// 56.5 ms of Krylov launches that way (plan_by_time: see the batch table in
+// DESIGN), four of 5 000 to 9 000 rows ran as three teams.
+static TeamPlan plan_launch(const std::vector<double> &work, const std::vector<int> &cap,
+                            const std::vector<int> &rows, int cmax, double scale) {
+  if (scale != 1.0) return plan_teams(work, cap, rows, cmax, scale);
+  double span;
+  return plan_by_time(work, cap, rows, cmax, &span);
+}
+
 // The planner on its own, for the host tests (no device work): the team of
 // every member and the plan's sizes.
 extern "C" int rbffd_plan_work_lists(int32_t m, const double *work, const int32_t *cap,
@@ -212,6 +316,33 @@ extern "C" int rbffd_plan_work_lists(int32_t m, const double *work, const int32_
     if (nctas) *nctas = T.nctas;
     if (team_size) *team_size = size;
     if (nteams) *nteams = teams;
+    return RBFFD_OK;
+  });
+}
+
+// The launches' own plan, for the host tests: each system's team and its
+// CTAs, and the modelled time of the longest team.
+extern "C" int rbffd_plan_teams(int32_t m, const double *work, const int32_t *cap,
+                                const int32_t *rows, int32_t cmax, int32_t *member_team,
+                                int32_t *member_ctas, int32_t *nctas, double *span) {
+  return guarded([&]() -> int {
+    if (m < 1 || cmax < 1 || !work || !cap || !rows || !member_team || !member_ctas)
+      return RBFFD_EINVAL;
+    for (int i = 0; i < m; ++i)
+      if (!(work[i] >= 0.0) || cap[i] < 1 || rows[i] < 1) return RBFFD_EINVAL;
+    double s;
+    const TeamPlan T =
+        plan_by_time(std::vector<double>(work, work + m), std::vector<int>(cap, cap + m),
+                     std::vector<int>(rows, rows + m), cmax, &s);
+    for (int i = 0; i < m; ++i) {
+      member_team[i] = -1;
+      member_ctas[i] = T.nb[i];
+    }
+    for (int t = 0; 4 * t < T.info_and_list[2]; ++t)
+      for (int k = T.info_and_list[4 * t + 2]; k < T.info_and_list[4 * t + 3]; ++k)
+        member_team[T.info_and_list[k]] = t;
+    if (nctas) *nctas = T.nctas;
+    if (span) *span = s;
     return RBFFD_OK;
   });
 }
@@ -280,7 +411,7 @@ static int launch_krylov(BatchScratch &S, int slot, int nr, std::vector<KrylovAr
   }
   std::vector<int> cap(m);
   for (int i = 0; i < m; ++i) cap[i] = args[i].nblocks;
-  const TeamPlan T = plan_teams(work, cap, rows, cmax, S.scale[slot]);
+  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot]);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
   KrylovArgs *hsys = (KrylovArgs *)(hb + S.off_sys[slot]);
@@ -319,7 +450,7 @@ static int launch_mixed(BatchScratch &S, int slot, int nr, int inner,
   }
   std::vector<int> cap(m);
   for (int i = 0; i < m; ++i) cap[i] = args[i].nblocks;
-  const TeamPlan T = plan_teams(work, cap, rows, cmax, S.scale[slot]);
+  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot]);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
   MixedArgs *hsys = (MixedArgs *)(hb + S.off_sys[slot]);
@@ -353,7 +484,8 @@ static int launch_fgmres(BatchScratch &S, int slot, std::vector<FgmresArgs> &arg
     set_error("batch: %d members exceed the %d co-resident CTAs of one launch", m, cmax);
     return RBFFD_EINVAL;
   }
-  const TeamPlan T = plan_teams(work, std::vector<int>(m, kdev::MAXB), rows, cmax, S.scale[slot]);
+  const TeamPlan T =
+      plan_launch(work, std::vector<int>(m, kdev::MAXB), rows, cmax, S.scale[slot]);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
   FgmresArgs *hsys = (FgmresArgs *)(hb + S.off_sys[slot]);

@@ -148,6 +148,8 @@ def load(path: str = LIB_PATH):
         "rbffd_batch_set_autotune": (C.c_int, [vp, C.c_int]),
         "rbffd_plan_work_lists": (C.c_int, [i32, vp, vp, vp, i32, dbl, C.POINTER(i32),
                                             C.POINTER(i32), C.POINTER(i32), vp]),
+        "rbffd_plan_teams": (C.c_int, [i32, vp, vp, vp, i32, vp, vp, C.POINTER(i32),
+                                       C.POINTER(dbl)]),
         "rbffd_server_create": (C.c_int, [vp, C.POINTER(ServerParams), C.POINTER(vp)]),
         "rbffd_server_submit": (C.c_int, [vp, C.POINTER(ProblemDesc), C.POINTER(SolveParams),
                                           C.POINTER(C.c_uint64)]),
@@ -528,6 +530,19 @@ def plan_work_lists(work, cap, rows, cmax, scale=1.0):
                                         float(scale), C.byref(nc), C.byref(ts), C.byref(nt),
                                         ptr(team)), "rbffd_plan_work_lists")
     return team, nc.value, ts.value, nt.value
+
+
+def plan_teams(work, cap, rows, cmax):
+    """The batched launches' plan (rbffd_plan_teams): (team of each solve, its
+    CTAs, CTAs in all, modelled time of the longest team)."""
+    work = np.ascontiguousarray(work, np.float64)
+    cap = np.ascontiguousarray(cap, np.int32)
+    rows = np.ascontiguousarray(rows, np.int32)
+    team, ctas = np.zeros(work.size, np.int32), np.zeros(work.size, np.int32)
+    nc, span = C.c_int32(0), C.c_double(0)
+    _check(load().rbffd_plan_teams(work.size, ptr(work), ptr(cap), ptr(rows), int(cmax), ptr(team),
+                                   ptr(ctas), C.byref(nc), C.byref(span)), "rbffd_plan_teams")
+    return team, ctas, nc.value, span.value
 
 
 def amg_aggregates_host(rowptr, col, val):
