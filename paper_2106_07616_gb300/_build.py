@@ -14,7 +14,7 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "librbffd.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 
-SOURCES = ["context.cu", "knn.cu", "weights.cu", "krylov.cu", "krylov_mixed.cu", "resident.cu", "ops.cu", "amg.cu",
+SOURCES = ["context.cu", "knn.cu", "weights.cu", "krylov.cu", "krylov_res.cu", "krylov_mixed.cu", "resident.cu", "ops.cu", "amg.cu",
            "amg_setup.cu", "fgmres.cu", "fgmres_res.cu",
            "problem.cu", "batch.cu", "server.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -38,6 +38,7 @@ struct KrylovArgs {
   int tpr;              // threads per row in the SpMV phases (1..8)
   int nblocks;          // CTAs that share the solve (batched launches)
   const AmgDev *amg;    // multigrid preconditioner (one RHS), or null: Jacobi
+  ResPlan res;          // resident solve (resident.cuh): team, halo lists (nb = 0: none)
 };
 
 constexpr int KB_NT = 256;  // threads per CTA of batched Krylov launches
@@ -100,6 +101,14 @@ int krylov_batch_max_ctas(rbffd_ctx *ctx, int nr);
 int krylov_batch_launch(rbffd_ctx *ctx, int nr, int nctas, const KrylovArgs *d_sys,
                         const int *d_cta_sys, const int *d_cta_first, bool amg = false);
 int krylov_launch(rbffd_ctx *ctx, int nr, int nblocks, const KrylovArgs &args);
+// The same solve on a resident team (krylov_res.cu), when the plan, the sizes
+// and, with a multigrid preconditioner, its hierarchy h allow it (*ran);
+// omega: level 0's smoothing weight; B: the dense coarse operator or null.
+constexpr int RES_DENSE64_N = 512;  // most level-1 rows of an FP64 dense coarse operator
+int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgDev *h,
+                      double omega, const double *B, bool *ran);
+int krylov_dense_ld(const AmgDev &h);
+int krylov_dense_build(rbffd_ctx *ctx, const AmgDev &h, double *B);
 size_t krylov_partials_doubles(int nr, int nblocks);
 
 }  // namespace rbffd

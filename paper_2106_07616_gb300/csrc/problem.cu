@@ -85,8 +85,9 @@ void free_amg(rbffd_problem *P) {
   P->fg_mem = nullptr;
   P->fg_bytes = 0;
   P->fgV = P->fgZ = nullptr;
-  if (P->fgB) dev_free(P->ctx, P->fgB, P->fgB_bytes);
+  if (P->fgB || P->amgB) dev_free(P->ctx, P->fgB ? (void *)P->fgB : P->amgB, P->fgB_bytes);
   P->fgB = nullptr;
+  P->amgB = nullptr;
   P->fgB_bytes = 0;
   P->fgR = nullptr;
   P->fgpart = nullptr;
@@ -280,6 +281,15 @@ void resident_args(rbffd_problem *P, MixedArgs *m) {
   m->pubv = P->mv[0].p0;
 }
 
+// An FP64 BiCGSTAB solve: on the resident team where it fits, else streaming.
+int issue_fp64(rbffd_problem *P, int nr, int nblocks, KrylovArgs &a) {
+  bool ran = false;
+  a.res = P->res;
+  RBFFD_TRY(krylov_res_launch(P->ctx, nr, a, a.amg ? &P->amg_host : nullptr,
+                              a.amg ? P->amg_info.omega[0] : 0.0, P->amgB, &ran));
+  return ran ? RBFFD_OK : krylov_launch(P->ctx, nr, nblocks, a);
+}
+
 // Issue the pressure-correction solve M x = b with the problem's p' solver
 // (no host synchronisation): flexible GMRES with the FP32 hierarchy,
 // mixed-precision Jacobi BiCGSTAB, or FP64 BiCGSTAB with the FP64
@@ -374,7 +384,15 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
   a.w[1] = P->kv[1];
   a.out = P->kout + 2;
   a.tpr = krylov_threads_per_row(P->n, 1, P->kblocks1);
-  return krylov_launch(ctx, 1, P->kblocks1, a);
+  if (a.amg) {
+    const int ld = P->res.nb > 0 && !P->amgB ? krylov_dense_ld(P->amg_host) : 0;
+    const size_t bytes = sizeof(double) * (size_t)ld * ld;
+    if (ld > 0 && dev_alloc(ctx, (void **)&P->amgB, bytes) == RBFFD_OK) {
+      P->fgB_bytes = bytes;
+      RBFFD_TRY(krylov_dense_build(ctx, P->amg_host, P->amgB));
+    }
+  }
+  return issue_fp64(P, 1, P->kblocks1, a);
 }
 
 // Issue one outer iteration (no host synchronisation beyond the first p'
@@ -469,20 +487,20 @@ int issue_outer(rbffd_problem *P, const rbffd_step_params *sp) {
     a.out = P->kout;
     a.tpr = krylov_threads_per_row(P->n, 2, P->kblocks2);
     if (!P->has_sym) {
-      RBFFD_TRY(krylov_launch(ctx, 2, P->kblocks2, a));
+      RBFFD_TRY(issue_fp64(P, 2, P->kblocks2, a));
     } else {
       KrylovArgs b1 = a;
       b1.b[1] = nullptr;
       b1.x[1] = nullptr;
       b1.tpr = krylov_threads_per_row(P->n, 1, P->kblocks1);
-      RBFFD_TRY(krylov_launch(ctx, 1, P->kblocks1, b1));
+      RBFFD_TRY(issue_fp64(P, 1, P->kblocks1, b1));
       b1.val = P->Am2;
       b1.dinv = P->m_dinv2;
       b1.b[0] = P->bv;
       b1.x[0] = P->vt;
       b1.w[0] = P->kv[1];
       b1.out = P->kout + 1;
-      RBFFD_TRY(krylov_launch(ctx, 1, P->kblocks1, b1));
+      RBFFD_TRY(issue_fp64(P, 1, P->kblocks1, b1));
     }
   }
   prof_end(ctx, 0);
@@ -678,7 +696,6 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       o_part32 = c.take<char>(krylov_ir_partials_inner_bytes(2, kb, P->inner));
     }
     size_t o_hl = 0, o_hi = 0, o_li = 0, o_rp = 0;
-    if (!mixed && d->precond != RBFFD_PRECOND_AMG_FGMRES) P->res.nb = 0;
     if (P->res.nb > 0) {
       o_hl = c.take<int32_t>((size_t)P->res.nb * P->res.hstride);
       o_hi = c.take<int32_t>(2 * (size_t)P->res.nb);

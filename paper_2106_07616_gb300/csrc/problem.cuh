@@ -109,7 +109,10 @@ struct rbffd_problem {
   float *fgV = nullptr, *fgZ = nullptr;       // FP32 basis and directions
   void *fgpart = nullptr;
   int fg_m = 0, fg_blocks = 0;
-  float *fgB = nullptr;  // dense coarse operator (fgmres_res.cu), or null
+  // dense coarse operator of the resident p' solve (fgmres_res.cu: FP32,
+  // krylov_res.cu: FP64), or null
+  float *fgB = nullptr;
+  double *amgB = nullptr;
   size_t fgB_bytes = 0;
 };
 

@@ -172,6 +172,8 @@ __device__ __forceinline__ bool team_barrier(Team &t) {
   return s_ok != 0;
 }
 
+// active: false when the whole warp's values are zero (it then spends no
+// arithmetic on them).
 // Totals over the team of V values per thread, into tot[0..V) (shared; all
 // threads may read it on return), with a team barrier on the way.  Sums run
 // in a fixed order: every CTA gets bit-identical totals.  wsum: V x 32
@@ -181,10 +183,11 @@ __device__ __forceinline__ bool team_barrier(Team &t) {
 // still reads these.
 template <int V, typename P>
 __device__ __forceinline__ bool team_totals(Team &t, P (&val)[pow2_ge(V)], P *tot, P *wsum,
-                                            P *cpart, P *gpart) {
+                                            P *cpart, P *gpart, bool active = true) {
   constexpr int VP = pow2_ge(V);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  warp_totals<V>(val);
+  if (active) warp_totals<V>(val);
+  else val[0] = P(0);
   if ((lane & (32 / VP - 1)) == 0 && lane / (32 / VP) < V)
     wsum[(lane / (32 / VP)) * 32 + w] = val[0];
   __syncthreads();

@@ -42,6 +42,8 @@ CASES = {
 OUTLET = ("symmetry", "last_cta_empty")
 RUNS = [(c, p, rbffd.PRECOND_AMG) for c in sorted(CASES)
         for p in (rbffd.PREC_MIXED, rbffd.PREC_MIXED_FF)]
+RUNS += [(c, rbffd.PREC_FP64, pc) for c in sorted(CASES)
+         for pc in (rbffd.PRECOND_JACOBI, rbffd.PRECOND_AMG)]
 RUNS += [(c, rbffd.PREC_MIXED, rbffd.PRECOND_AMG_FGMRES) for c in sorted(CASES)
          if c not in OUTLET]
 
