@@ -34,6 +34,10 @@ struct rbffd_ctx {
   // flexible GMRES's Gram-Schmidt (rbffd_ctx_set_fgmres_reorth): 0 one
   // pass, 1 two passes a step, 2 two passes with the second delayed
   int fgmres_reorth = 1;
+  // device workspace of the calls that need one for their own duration
+  // (ctx_scratch), freed with the context
+  void *scratch = nullptr;
+  size_t scratch_bytes = 0;
   // pinned host scratch for small read-backs
   void *pinned = nullptr;
   size_t pinned_bytes = 0;
@@ -110,6 +114,11 @@ void dev_free(rbffd_ctx *ctx, void *p, size_t bytes);
 // the error text is set) / give them back
 bool dev_reserve(rbffd_ctx *ctx, size_t bytes);
 void dev_release(rbffd_ctx *ctx, size_t bytes);
+// Device workspace of at least `bytes`, valid until the next call on the
+// context (its calls are serialised, and each waits for its own kernels).
+// Kept between calls -- cudaMalloc and cudaFree cost 0.1 ms and more a call --
+// up to 64 MB; a larger one replaces it and is given back at the next call.
+int ctx_scratch(rbffd_ctx *ctx, size_t bytes, void **out);
 // Small pinned host buffer of at least `bytes` (owned by the context).
 int pinned(rbffd_ctx *ctx, size_t bytes, void **out);
 

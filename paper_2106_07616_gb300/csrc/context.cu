@@ -51,6 +51,21 @@ void dev_free(rbffd_ctx *ctx, void *p, size_t bytes) {
   dev_release(ctx, bytes);
 }
 
+int ctx_scratch(rbffd_ctx *ctx, size_t bytes, void **out) {
+  *out = nullptr;
+  constexpr size_t KEEP = (size_t)64 << 20;
+  if (ctx->scratch_bytes < bytes || (ctx->scratch_bytes > KEEP && bytes <= KEEP)) {
+    cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, ctx->scratch, ctx->scratch_bytes);
+    ctx->scratch = nullptr;
+    ctx->scratch_bytes = 0;
+    RBFFD_TRY(dev_alloc(ctx, &ctx->scratch, bytes));
+    ctx->scratch_bytes = bytes;
+  }
+  *out = ctx->scratch;
+  return RBFFD_OK;
+}
+
 int pinned(rbffd_ctx *ctx, size_t bytes, void **out) {
   if (ctx->pinned_bytes < bytes) {
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
@@ -110,6 +125,7 @@ static void ctx_free(rbffd_ctx *ctx) {
   cudaSetDevice(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
+  if (ctx->scratch) cudaFree(ctx->scratch);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
   for (int k = 0; k < 8; ++k)
     if (ctx->ev[k]) cudaEventDestroy(ctx->ev[k]);

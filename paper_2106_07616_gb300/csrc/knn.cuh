@@ -7,8 +7,9 @@
 namespace rbffd {
 
 struct KnnLayout {
-  int G, m;
-  size_t off_bbox, off_err, off_cell, off_cnt, off_start, off_cursor, off_pts;
+  int m;              // cells at most
+  size_t off_bbox, off_cnt, off_cell, off_start, off_pts;
+  size_t zero_bytes;  // the first bytes, zeroed before a search
   size_t bytes;
 };
 
