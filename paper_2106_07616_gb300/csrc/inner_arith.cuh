@@ -64,6 +64,12 @@ __device__ __forceinline__ ff ff_from_double(double v) {
 
 __device__ __forceinline__ double ff_to_double(ff v) { return (double)v.hi + (double)v.lo; }
 
+// a b as an unevaluated sum of two FP32 numbers, exactly
+__device__ __forceinline__ ff ff_two_prod(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return {p, __fmaf_rn(a, b, -p)};
+}
+
 struct ArithF32 {
   using S = float;   // stored values (matrix, vectors)
   using A = float;   // accumulators

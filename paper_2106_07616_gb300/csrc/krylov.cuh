@@ -74,6 +74,8 @@ struct MixedArgs {
   double inner_tol;      // relative reduction asked of each inner solve
   int inner_maxit;       // cap on inner iterations per sweep
   int max_sweeps;
+  int ff_sums;           // resident solve: products summed in float-float (p')
+  int o_xold;            // resident solve: its place for x before a sweep
   // resident solve (resident.cuh): the team and its halo lists (nb = 0: none),
   // and the vectors published to the other CTAs, n x NR values side by side
   ResPlan res;

@@ -587,13 +587,18 @@ __global__ void __launch_bounds__(NT) k_bicgstab_ir(MixedArgs A) {
 //            p = r + beta (p - omega v) follow on the spot),
 //   phase C: v of this one (s = r - alpha v follows),
 // one load an entry of the list instead of up to five a matrix entry or
-// window entry.  What bounds it: the exchange (about 1.2 us over the grid,
+// window entry.  A sweep that leaves a larger FP64 residual than it started
+// from is undone and made again with another shadow residual (r^_i = r_i (1 +
+// h_i / 2), h a hash of the row and the attempt): the FP32 recurrences of
+// badly conditioned p' systems stall or run away on some rounding.  What bounds it: the exchange (about 1.2 us over the grid,
 // twice an iteration) and the halo's round trip.
 // Measured on GB300, a whole outer iteration with the streaming solve and
 // with this one (the p' solve the same): cavity 200^2 (q = 30, two right-hand
 // sides) 12.5 -> 8.4 ms, cylinder 147 827 (q = 20, two single solves)
 // 20.2 -> 11.6 ms, Kovasznay 50^2 (one cluster) 6.9 -> 4.9 ms.
 namespace {
+
+constexpr int IR_TRIES = 3;  // attempts in a row to redo a sweep that made things worse
 
 // What every thread of the CTA needs of the recurrences' scalars, and the
 // scalars themselves.  rho, alpha and omega are float-float: an FP64
@@ -608,6 +613,10 @@ struct IrCoef {
   int run[NR], fin[NR], any;
   ff rho[NR], alpha[NR];
   float lim2[NR], big2[NR];  // (inner_tol r0)^2, (1e3 r0)^2 of the sweep
+  double rr[NR];             // |r|^2 the sweep started from
+  // the sweep made the residual worse; its iterate was restored and its residual
+  // is being formed again; how often in a row
+  int undo[NR], undone[NR], tries[NR];
   int it[NR], inner_it[NR];
 };
 
@@ -615,23 +624,30 @@ __device__ __forceinline__ ff ff_of(float v) { return ff(v, 0.f); }
 __device__ __forceinline__ ff ff_of(ff v) { return v; }
 __device__ __forceinline__ void coef_of(ff v, float &o) { o = v.hi; }
 __device__ __forceinline__ void coef_of(ff v, ff &o) { o = v; }
+__device__ __forceinline__ void prod(float &o, float a, float b) { o = __fmul_rn(a, b); }
+__device__ __forceinline__ void prod(ff &o, float a, float b) { o = ff_two_prod(a, b); }
+__device__ __forceinline__ void prod(ff &o, ff a, ff b) { o = ff_mul(a, b); }
 __device__ __forceinline__ ff ff_div(ff a, ff b) {
   const float q = __fdiv_rn(a.hi, b.hi);
   const ff r = ff_add(a, ff_neg(ff_mul(b, ff(q, 0.f))));
   return ff_fast_two_sum(q, __fdiv_rn(r.hi, b.hi));
 }
 
-template <int NR, class IA, int E>
+// PT: partial sums of the products, the inner arithmetic's own or, for the
+// Jacobi-scaled p' systems (FF sums), float-float: their FP32 recurrences
+// converge or stall on the products' rounding (of 24 clouds of 900 points
+// four iterations each, 4 stalled with FP32 sums and 2 with float-float ones),
+// while the momentum systems gain nothing for the 5 % of time the sums cost.
+template <int NR, class IA, int E, class PT>
 __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
   using S = typename IA::S;
-  using PT = typename IA::P;
   using V = res::Vec<S, NR>;
   constexpr int ES = (int)sizeof(V);
   __shared__ PT wsum[5 * NR * 32];
   __shared__ PT cpart[2 * 5 * NR * RES_CLUSTER];
-  __shared__ double wsum64[2 * NR * 32], cpart64[2 * 2 * NR * RES_CLUSTER];
+  __shared__ double wsum64[3 * NR * 32], cpart64[2 * 3 * NR * RES_CLUSTER];
   __shared__ PT tot[5 * NR];
-  __shared__ double tot64[2 * NR];
+  __shared__ double tot64[3 * NR];
   __shared__ IRS ks[NR];
   __shared__ IrCoef<NR, IA> co;
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -646,6 +662,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
   S *dinv = reinterpret_cast<S *>(d + R);
   int *list = reinterpret_cast<int *>(dinv + hm);
   double *xs = reinterpret_cast<double *>(dyn);
+  double *xold = reinterpret_cast<double *>(dyn + A.o_xold);  // x before the sweep, own rows
   V *pubt = reinterpret_cast<V *>(A.pubt), *pubv = reinterpret_cast<V *>(A.pubv);
   const S *val = reinterpret_cast<const S *>(A.valin);
   for (int e = tid; e < L; e += RES_NT) {
@@ -671,6 +688,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
     c.state = KRY_RUNNING;
     c.sweeps = c.it = c.inner_it = 0;
     c.in_sweep = c.inner = c.half = c.zero = 0;
+    co.undo[tid] = co.undone[tid] = co.tries[tid] = 0;
   }
   // every CTA of a cluster has started before any writes to another
   bool ok = true;
@@ -729,9 +747,9 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
         const double s = ax[k];
         for (int u = 1; u < T; ++u) ax[k] += __shfl_sync(0xffffffffu, s, (lane + u) & 31);
       }
-      double acc[res::pow2_ge(2 * NR)];
+      double acc[res::pow2_ge(3 * NR)];
 #pragma unroll
-      for (int k = 0; k < res::pow2_ge(2 * NR); ++k) acc[k] = 0.0;
+      for (int k = 0; k < res::pow2_ge(3 * NR); ++k) acc[k] = 0.0;
       if (row.lead) {
         V rf;
 #pragma unroll
@@ -740,13 +758,18 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           rf.x[k] = IA::from_double(ri);
           if (part[k]) {
             rh[k] = rf.x[k];
-            acc[2 * k] = bi * bi;
-            acc[2 * k + 1] = ri * ri;
+            if (co.tries[k] > 0) {
+              const uint32_t h = mis_hash((uint32_t)row.i * 31u + (uint32_t)co.tries[k]);
+              rh[k] = IA::from_double(ri * (1.0 + ((double)h * 0x1p-32 - 0.5)));
+            }
+            acc[3 * k] = bi * bi;
+            acc[3 * k + 1] = ri * ri;
+            acc[3 * k + 2] = ri * IA::to_double(rh[k]);
           }
         }
         pubt[row.i] = rf;
       }
-      ok = res::team_totals<2 * NR>(team, acc, tot64, wsum64, cpart64,
+      ok = res::team_totals<3 * NR>(team, acc, tot64, wsum64, cpart64,
                                      reinterpret_cast<double *>(A.res.part));
       if (!ok) break;
       if (tid == 0) {
@@ -758,23 +781,39 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           c.inner = 0;
           c.zero = 0;
           if (part[k]) {
-            if (c.sweeps == 0) c.bnorm = sqrt(tot64[2 * k]);
+            if (c.sweeps == 0) c.bnorm = sqrt(tot64[3 * k]);
             if (c.bnorm == 0.0) {
               c.relres = 0.0;
               c.state = KRY_OK;
               c.zero = 1;
             } else {
-              const double rr = tot64[2 * k + 1];
+              const double rr = tot64[3 * k + 1];
+              const bool worse = c.sweeps > 0 && !(rr <= co.rr[k]);
               c.relres = sqrt(rr) / c.bnorm;
-              if (!(c.relres == c.relres)) c.state = KRY_DIVERGED;
+              co.undo[k] = 0;
+              if (worse && !(c.relres <= A.tol) && c.sweeps < A.max_sweeps && c.it < A.maxit &&
+                  !co.undone[k] && co.tries[k] < IR_TRIES) {
+                // back to the iterate before the sweep; its residual again
+                co.undo[k] = 1;
+                co.undone[k] = 1;
+                co.tries[k]++;
+                any = 1;
+              } else if (!(c.relres == c.relres)) c.state = KRY_DIVERGED;
               else if (c.relres <= A.tol) c.state = KRY_OK;
               else if (c.sweeps >= A.max_sweeps || c.it >= A.maxit) c.state = KRY_NOCONV;
               else {
                 c.in_sweep = 1;
                 c.inner = 1;
-                co.rho[k] = ff_from_double(rr);
+                co.rho[k] = ff_from_double(tot64[3 * k + 2]);
+                if (!co.undone[k]) co.tries[k] = 0;
+                co.undone[k] = 0;
+                co.rr[k] = rr;
                 co.lim2[k] = (float)(A.inner_tol * A.inner_tol * rr);
-                co.big2[k] = (float)(1e6 * rr);
+                // |r| may grow 1e3-fold, and as much again with every attempt:
+                // some recurrences pass a larger hump on their way
+                double grow = 1e6;
+                for (int t = 0; t < co.tries[k]; ++t) grow *= 1e6;
+                co.big2[k] = (float)(grow * rr);
                 any = 1;
               }
             }
@@ -793,6 +832,18 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           for (int i = r0 + tid; i < r1; i += RES_NT) A.x[k][i] = 0.0;
         }
       if (!co.any) break;
+      bool undo = false;
+#pragma unroll
+      for (int k = 0; k < NR; ++k)
+        if (co.undo[k]) {
+          undo = true;
+          for (int e = tid; e < r1 - r0; e += RES_NT) A.x[k][r0 + e] = xold[NR * e + k];
+        }
+      if (undo) {
+        // the systems not undone take their turn after it, from the same x
+        if (!res::team_barrier(team)) { ok = false; break; }
+        continue;
+      }
       for (int e = tid; e < R; e += RES_NT) {
 #pragma unroll
         for (int k = 0; k < NR; ++k) d[e].x[k] = IA::szero();
@@ -854,13 +905,10 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
 #pragma unroll
           for (int k = 0; k < NR; ++k) {
             vn.x[k] = IA::from_acc(av[k]);
-            typename IA::A x = IA::zero(), y = IA::zero();
             if (run[k]) {
-              IA::madd(x, rh[k], vn.x[k]);
-              IA::madd(y, ri.x[k], ri.x[k]);
+              prod(acc[2 * k], rh[k], vn.x[k]);
+              prod(acc[2 * k + 1], ri.x[k], ri.x[k]);
             }
-            acc[2 * k] = IA::part(x);
-            acc[2 * k + 1] = IA::part(y);
           }
           pubv[row.i] = vn;
         }
@@ -928,16 +976,11 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
             tn.x[k] = IA::from_acc(at[k]);
             if (run[k]) {
               const S s = si.x[k], t = tn.x[k];
-              typename IA::A z[5];
-#pragma unroll
-              for (int m = 0; m < 5; ++m) z[m] = IA::zero();
-              IA::madd(z[0], s, s);
-              IA::madd(z[1], t, t);
-              IA::madd(z[2], t, s);
-              IA::madd(z[3], rh[k], s);
-              IA::madd(z[4], rh[k], t);
-#pragma unroll
-              for (int m = 0; m < 5; ++m) acc[5 * k + m] = IA::part(z[m]);
+              prod(acc[5 * k], s, s);
+              prod(acc[5 * k + 1], t, t);
+              prod(acc[5 * k + 2], t, s);
+              prod(acc[5 * k + 3], rh[k], s);
+              prod(acc[5 * k + 4], rh[k], t);
             }
           }
           pubt[row.i] = tn;
@@ -1008,8 +1051,11 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
 #pragma unroll
     for (int k = 0; k < NR; ++k)
       if (ks[k].in_sweep) {
-        for (int e = tid; e < r1 - r0; e += RES_NT)
-          A.x[k][r0 + e] = A.x[k][r0 + e] + IA::to_double(d[e].x[k]);
+        for (int e = tid; e < r1 - r0; e += RES_NT) {
+          const double x = A.x[k][r0 + e];
+          xold[NR * e + k] = x;
+          A.x[k][r0 + e] = x + IA::to_double(d[e].x[k]);
+        }
       }
     __syncthreads();
     if (tid < NR && ks[tid].in_sweep) {
@@ -1029,26 +1075,34 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
   }
 }
 
-template <int NR, class IA>
+template <int NR, class IA, class PT>
 const void *ir_res_fn(int E) {
-  if (E <= 6) return (const void *)k_ir_res<NR, IA, 6>;
-  if (E <= 12) return (const void *)k_ir_res<NR, IA, 12>;
+  if (E <= 6) return (const void *)k_ir_res<NR, IA, 6, PT>;
+  if (E <= 12) return (const void *)k_ir_res<NR, IA, 12, PT>;
   if constexpr (sizeof(typename IA::S) == 4)
-    if (E <= 24) return (const void *)k_ir_res<NR, IA, 24>;
+    if (E <= 24) return (const void *)k_ir_res<NR, IA, 24, PT>;
   return nullptr;
+}
+
+// shared memory before x's own rows: the halo's vectors, d, 1 / d, the list
+size_t ir_res_halo_bytes(size_t s, int nr, const ResPlan &p) {
+  return (4 * s * nr * p.hmax + s * nr * p.R + s * p.hmax + 4 * (size_t)p.hmax + 31) / 16 * 16;
 }
 
 // the kernel and its shared memory for a plan, or null: the rows' entries do
 // not fit the registers, or the halo not the shared memory
-const void *ir_res_kernel(int nr, int inner, int q, const ResPlan &p, size_t *smem) {
+const void *ir_res_kernel(int nr, int inner, bool ff_sums, int q, const ResPlan &p,
+                          size_t *smem) {
   if (p.nb < 1 || p.hmax < 1 || p.hmax > p.hstride) return nullptr;
   const int E = (q + p.T - 1) / p.T;
   const size_t s = inner == INNER_FF ? 8 : 4;
   if (s * nr * p.hmax > 65535) return nullptr;
-  *smem = 4 * s * nr * p.hmax + s * nr * p.R + s * p.hmax + 4 * (size_t)p.hmax + 16;
+  *smem = ir_res_halo_bytes(s, nr, p) + 8 * (size_t)nr * p.R;
   if (*smem > 200 * 1024) return nullptr;
-  if (inner == INNER_FF) return nr == 1 ? ir_res_fn<1, ArithFF>(E) : ir_res_fn<2, ArithFF>(E);
-  return nr == 1 ? ir_res_fn<1, ArithF32>(E) : ir_res_fn<2, ArithF32>(E);
+  if (inner == INNER_FF)
+    return nr == 1 ? ir_res_fn<1, ArithFF, ff>(E) : ir_res_fn<2, ArithFF, ff>(E);
+  if (nr == 2) return ir_res_fn<2, ArithF32, float>(E);
+  return ff_sums ? ir_res_fn<1, ArithF32, ff>(E) : ir_res_fn<1, ArithF32, float>(E);
 }
 
 }  // namespace
@@ -1056,11 +1110,12 @@ const void *ir_res_kernel(int nr, int inner, int q, const ResPlan &p, size_t *sm
 // Runs the resident kernel when the plan and sizes allow it (*ran = true).
 static int ir_res_launch(rbffd_ctx *ctx, int nr, const MixedArgs &args, bool *ran) {
   size_t smem = 0;
-  const void *fn = ir_res_kernel(nr, args.inner, args.q, args.res, &smem);
+  const void *fn = ir_res_kernel(nr, args.inner, args.ff_sums != 0, args.q, args.res, &smem);
   *ran = fn != nullptr;
   if (!fn) return RBFFD_OK;
   MixedArgs a = args;
   a.tpr = args.res.T;
+  a.o_xold = (int)ir_res_halo_bytes(args.inner == INNER_FF ? 8 : 4, nr, args.res);
   RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
   if (!args.res.cluster) RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
   return res_launch(ctx, args.res, fn, &a, smem, "k_ir_res");

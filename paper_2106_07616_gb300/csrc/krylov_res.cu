@@ -32,10 +32,18 @@ namespace {
 // restarts from the best iterate, restarts after a breakdown.
 constexpr double BLOWUP2 = 1e20;  // squared
 constexpr int MAX_BLOWUPS = 8, MAX_BREAKDOWNS = 3;
+// A solve of CHECK_ITS iterations or more whose recurrence meets the tolerance
+// is checked against its true residual, and restarted from there where that
+// is over CHECK2^(1/2) times the tolerance, at most MAX_CHECKS times: after
+// thousands of iterations the two part (a 19 920-row channel, 7 257 Jacobi
+// iterations to 1e-12: fields 1.4e-8 off, against 4e-11 with a restart).
+constexpr double CHECK2 = 100.0;
+constexpr int MAX_CHECKS = 3, CHECK_ITS = 1000;
 
 struct Scalars {
   double bnorm, tol2, rho, alpha, omega, beta, rr, best2, relres;
   int it, restarts, blowups, state, need_init, restore, save, run, first, half;
+  int checks, met;  // true-residual checks made; the recurrence met the tolerance
 };
 
 struct BicgResArgs {
@@ -161,7 +169,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
     c.bnorm = c.rho = c.alpha = c.omega = 1.0;
     c.beta = c.relres = c.rr = c.tol2 = 0.0;
     c.best2 = 1e308;
-    c.it = c.restarts = c.blowups = c.restore = c.save = c.half = 0;
+    c.it = c.restarts = c.blowups = c.restore = c.save = c.half = c.checks = c.met = 0;
     c.state = KRY_RUNNING;
     c.need_init = c.first = c.run = 1;
   }
@@ -312,6 +320,15 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
     return res::team_barrier(team);
   };
 
+  // the recurrence has met the tolerance (thread k)
+  auto met = [&](Scalars &c) {
+    if (c.checks >= MAX_CHECKS || c.it < CHECK_ITS) {
+      c.state = KRY_OK;
+    } else {
+      c.checks++;
+      c.met = c.need_init = 1;
+    }
+  };
   // a system whose recurrence ran away (or became non-finite) restarts from
   // its best iterate, a bounded number of times (thread k)
   auto blowup = [&](Scalars &c, int final_state) {
@@ -373,9 +390,16 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
           c.bnorm = sqrt(bb);
           c.tol2 = K.tol * K.tol * bb;
         }
-        c.rr = rr;
         c.first = 1;
-        if (c.bnorm == 0.0) {
+        if (c.met) {
+          c.met = 0;
+          c.best2 = 1e308;
+          // the recurrence's residual is reported, as without the check
+          if (rr <= CHECK2 * c.tol2) c.state = KRY_OK;
+        }
+        if (c.state == KRY_RUNNING) c.rr = rr;
+        if (c.state == KRY_OK) {
+        } else if (c.bnorm == 0.0) {
           c.rr = 0.0;
           c.state = KRY_OK;
           c.half = 3;  // x = 0
@@ -505,7 +529,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
         if (!isfinite(rr)) {
           blowup(c, KRY_DIVERGED);
         } else if (rr <= c.tol2) {
-          c.state = KRY_OK;
+          met(c);
         } else {
           bool go = true;
           if (rr < c.best2) {
@@ -629,7 +653,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
           } else if (ss <= c.tol2) {
             c.half = 1;
             c.rr = ss;
-            c.state = KRY_OK;
+            met(c);
           } else {
             c.omega = tt == 0.0 ? 0.0 : om0;
             const double rho_new = rhs - c.omega * rht;

@@ -359,6 +359,7 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
     m.b[0] = b;
     m.x[0] = x;
     m.w[0] = P->mv[0];
+    m.ff_sums = 1;
     resident_args(P, &m);
     m.out = P->kout + 2;
     m.tpr = krylov_threads_per_row(P->n, 1, P->kblocks1);
