@@ -550,8 +550,9 @@ int rbffd_plan_work_lists(int32_t m, const double *work, const int32_t *cap, con
                           int32_t cmax, double scale, int32_t *nctas, int32_t *team_size,
                           int32_t *nteams, int32_t *member_team);
 
-/* The plan the batched launches use (host only): as rbffd_plan_work_lists,
- * but the teams differ in size, chosen so that the team that finishes last
+/* The plan the batched streaming launches use where its span is a fifth
+ * shorter than that of equal teams (host only): as rbffd_plan_work_lists, but
+ * the teams differ in size, chosen so that the team that finishes last
  * finishes soonest, a solve of rows r and work w on c CTAs taking
  * (w / r) (512 + r / c).  Solve i goes to team member_team[i] of
  * member_ctas[i] CTAs (at most cap[i], and what 8 threads a row fill);

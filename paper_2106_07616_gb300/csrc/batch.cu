@@ -102,7 +102,8 @@ int BatchScratch::reserve(rbffd_ctx *c, int members) {
     return a;
   };
   for (int k = 0; k < NSLOT; ++k) {
-    off_sys[k] = take(std::max({sizeof(KrylovArgs), sizeof(FgmresArgs), sizeof(MixedArgs)}) * cap);
+    off_sys[k] = take(std::max({sizeof(KrylovArgs), sizeof(FgmresArgs), sizeof(MixedArgs),
+                                krylov_res_args_bytes()}) * cap);
     off_cta_sys[k] = take(sizeof(int) * maxc);
     team_words = 4 * maxc + cap;
     off_cta_first[k] = take(sizeof(int) * team_words);
@@ -280,17 +281,182 @@ static TeamPlan plan_by_time(const std::vector<double> &work, const std::vector<
   return best;
 }
 
-// The plan a launch takes: by time, or, for the autotuner's other scales, the
-// equal teams of plan_teams.  Why: equal teams are as small as the smallest
-// member's partial sums allow (23 CTAs for 1 444 rows), and members beyond
-// the teams wait for their turn; 16 members of 1 444 to 50 625 rows took
-// 56.5 ms of Krylov launches that way (plan_by_time: see the batch table in
-// DESIGN), four of 5 000 to 9 000 rows ran as three teams.
+// The plan a launch takes: by time where that is a fifth shorter than equal
+// teams, else (and for the autotuner's other scales) the equal teams of
+// plan_teams.  Why: equal teams are as small as the smallest member's partial
+// sums allow (23 CTAs for 1 444 rows), and members beyond the teams wait for
+// their turn; 16 members of 1 444 to 50 625 rows took 56.5 ms of Krylov
+// launches that way and 44.0 ms by time (span: less than half).  256 members
+// average out: the span by time is 6% shorter, but the time was 5 to 7% longer
+// (0.89 against 0.95 ns a row and p' iteration: the cost leaves out what many
+// teams at once cost in L2).  *span: of the plan, in the cost's units.
 static TeamPlan plan_launch(const std::vector<double> &work, const std::vector<int> &cap,
-                            const std::vector<int> &rows, int cmax, double scale) {
-  if (scale != 1.0) return plan_teams(work, cap, rows, cmax, scale);
-  double span;
-  return plan_by_time(work, cap, rows, cmax, &span);
+                            const std::vector<int> &rows, int cmax, double scale, double *span) {
+  TeamPlan E = plan_teams(work, cap, rows, cmax, scale);
+  *span = 0.0;
+  for (int t = 0; 4 * t < E.info_and_list[2]; ++t) {
+    double time = 0.0;
+    for (int k = E.info_and_list[4 * t + 2]; k < E.info_and_list[4 * t + 3]; ++k) {
+      const int i = E.info_and_list[k];
+      time += work[i] / rows[i] * PLAN_LATENCY_ROWS + work[i] / E.nb[i];
+    }
+    *span = std::max(*span, time);
+  }
+  if (scale != 1.0) return E;
+  double s;
+  TeamPlan T = plan_by_time(work, cap, rows, cmax, &s);
+  if (s > 0.8 * *span) return E;
+  *span = s;
+  return T;
+}
+
+// ---- resident teams (krylov_res.cu) -----------------------------------------
+
+// Time of a resident iteration in us: fixed cost, then per row of a CTA and
+// per matrix entry of a CTA's row.  From single solves of 1 444 to 50 625 rows
+// (q = 12 to 42): 36 to 87 us with the multigrid cycle, 19 to 41 us for the
+// momentum pair.
+struct ResCost {
+  double fixed, row, entry;
+};
+constexpr ResCost RES_COST[2] = {{20.0, 0.002, 0.0013}, {38.0, 0.040, 0.0024}};
+// A unit of plan_by_time's spans (a row of a 256-thread CTA) in us per entry
+// of the row: launches of 16 members (q = 12 to 42) and of four (q = 20, 30).
+constexpr double STREAM_UNIT[2] = {0.0020, 0.0052};
+
+// Members of more rows in all than this (half of what a chip of 1024-thread
+// CTAs holds) leave teams of barely their least size, and teams in turn: not
+// tried (16 members of 279 000 rows: 33.6 ms planned, 27.4 ms streaming).
+static double resident_rows(const rbffd_ctx *ctx) { return 0.5 * RES_NT * ctx->num_sms; }
+
+struct ResMember {
+  double its;       // expected iterations
+  int rows, q;
+  int lo, hi;       // first and last team size (of RES_SIZES) that fits
+};
+
+// The resident launch's teams: the shortest span at which the members,
+// largest least team first, find room -- in a team that is there, enlarged if
+// need be, or a new one, whichever takes the fewest CTAs -- by bisection; then
+// the CTAs left go to the slowest teams.  Members of unlike size share the
+// chip as teams of their own.
+// *time_us: the span (1e300: no plan).
+static TeamPlan plan_resident(const std::vector<ResMember> &mem, bool amg, int cmax,
+                              double *time_us) {
+  const int m = (int)mem.size();
+  const ResCost c = RES_COST[amg];
+  std::vector<double> fixed(m), work(m);
+  std::vector<int> order(m);
+  double total = 0.0;
+  for (int i = 0; i < m; ++i) {
+    fixed[i] = mem[i].its * c.fixed;
+    work[i] = mem[i].its * mem[i].rows * (c.row + c.entry * mem[i].q);
+    total += fixed[i] + work[i];
+  }
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    return mem[a].lo != mem[b].lo ? mem[a].lo > mem[b].lo : work[a] > work[b];
+  });
+  struct Team {
+    double fixed = 0.0, work = 0.0;
+    int k = 0, hi = RES_NSIZES - 1;
+    std::vector<int> list;
+    double time(int j) const { return fixed + work / RES_SIZES[j]; }
+  };
+  auto pack = [&](double span, std::vector<Team> &G) {
+    G.clear();
+    int left = cmax;
+    for (int i : order) {
+      int at = -1, size = 0, extra = left + 1;
+      for (int t = 0; t <= (int)G.size(); ++t) {
+        const bool open = t == (int)G.size();
+        const double f = fixed[i] + (open ? 0.0 : G[t].fixed),
+                     w = work[i] + (open ? 0.0 : G[t].work);
+        const int hi = open ? mem[i].hi : std::min(G[t].hi, mem[i].hi);
+        const int have = open ? 0 : RES_SIZES[G[t].k];
+        for (int k = open ? mem[i].lo : std::max(G[t].k, mem[i].lo); k <= hi; ++k) {
+          if (RES_SIZES[k] - have >= extra) break;
+          if (f + w / RES_SIZES[k] > span) continue;
+          at = t;
+          size = k;
+          extra = RES_SIZES[k] - have;
+          break;
+        }
+      }
+      if (at < 0) return false;
+      if (at == (int)G.size()) G.emplace_back();
+      Team &g = G[at];
+      g.fixed += fixed[i];
+      g.work += work[i];
+      g.hi = std::min(g.hi, mem[i].hi);
+      g.k = size;
+      g.list.push_back(i);
+      left -= extra;
+    }
+    return true;
+  };
+  std::vector<Team> G, H;
+  double lo = 0.0, hi = total;  // every member in turn on one CTA
+  *time_us = 1e300;
+  TeamPlan T;
+  if (!pack(hi, G)) return T;
+  for (int r = 0; r < 24 && hi - lo > 0.01 * hi; ++r) {
+    const double mid = 0.5 * (lo + hi);
+    if (pack(mid, H)) {
+      hi = mid;
+      std::swap(G, H);
+    } else {
+      lo = mid;
+    }
+  }
+  const int ng = (int)G.size();
+  int left = cmax;
+  for (const Team &g : G) left -= RES_SIZES[g.k];
+  std::vector<int> heap(ng);
+  std::iota(heap.begin(), heap.end(), 0);
+  auto faster = [&](int a, int b) { return G[a].time(G[a].k) < G[b].time(G[b].k); };
+  std::make_heap(heap.begin(), heap.end(), faster);
+  *time_us = 0.0;
+  while (!heap.empty()) {
+    std::pop_heap(heap.begin(), heap.end(), faster);
+    Team &g = G[heap.back()];
+    const int more = g.k < g.hi ? RES_SIZES[g.k + 1] - RES_SIZES[g.k] : left + 1;
+    if (more <= left) {
+      ++g.k;
+      left -= more;
+      std::push_heap(heap.begin(), heap.end(), faster);
+    } else {
+      *time_us = std::max(*time_us, g.time(g.k));
+      heap.pop_back();
+    }
+  }
+  T.info_and_list.assign(4 * ng, 0);
+  T.nb.assign(m, 1);
+  for (int t = 0; t < ng; ++t) {
+    const int nb = RES_SIZES[G[t].k];
+    T.info_and_list[4 * t] = T.nctas;
+    T.info_and_list[4 * t + 1] = nb;
+    T.info_and_list[4 * t + 2] = (int)T.info_and_list.size();
+    for (int i : G[t].list) {
+      T.nb[i] = nb;
+      T.info_and_list.push_back(i);
+    }
+    T.info_and_list[4 * t + 3] = (int)T.info_and_list.size();
+    T.nctas += nb;
+    T.cta_team.resize(T.nctas, t);
+  }
+  return T;
+}
+
+// The team of system a (problem Q) at size k of RES_SIZES.
+static KrylovArgs at_size(const KrylovArgs &a, const rbffd_problem *Q, int k) {
+  KrylovArgs r = a;
+  const int nb = RES_SIZES[k];
+  r.res = ResPlan();
+  r.res.nb = nb;
+  r.res.R = (a.n + nb - 1) / nb;
+  r.res.hmax = Q->res_hm[k];
+  return r;
 }
 
 // The planner on its own, for the host tests (no device work): the team of
@@ -396,12 +562,76 @@ static int tpr_for(int n, int nb) {
   return T;
 }
 
+// The launch on resident teams, where every system fits one and their plan is
+// shorter than limit_us.
+static int launch_resident(BatchScratch &S, int slot, int nr, const std::vector<KrylovArgs> &args,
+                           const std::vector<double> &work, const std::vector<int> &rows,
+                           const std::vector<const rbffd_problem *> &probs, bool amg,
+                           double limit_us, bool *ran) {
+  rbffd_ctx *ctx = S.ctx;
+  const int m = (int)args.size();
+  *ran = false;
+  auto member_args = [&](int i, const KrylovArgs &a, void *out, size_t *smem) {
+    return krylov_res_args(nr, a, amg ? &probs[i]->amg_host : nullptr,
+                           amg ? probs[i]->amg_info.omega[0] : 0.0, probs[i]->amgB, out, smem);
+  };
+  std::vector<ResMember> mem(m);
+  const ResCost c = RES_COST[amg];
+  double least = 0.0;  // CTA-time no plan can do without
+  size_t smem = 0, need;
+  for (int i = 0; i < m; ++i) {
+    if (!probs[i]->res_hm_known) return RBFFD_OK;
+    ResMember &r = mem[i];
+    r = {work[i] / rows[i], rows[i], args[i].q, 0, -1};
+    for (int k = 0; k < RES_NSIZES; ++k) {
+      const int hm = probs[i]->res_hm[k];
+      if (hm > 0 && hm < 65536 && member_args(i, at_size(args[i], probs[i], k), nullptr, &need)) {
+        if (r.hi < 0) r.lo = k;
+        r.hi = k;
+      } else if (r.hi >= 0) {
+        break;
+      }
+    }
+    if (r.hi < 0) return RBFFD_OK;
+    least += r.its * (c.fixed * RES_SIZES[r.lo] + r.rows * (c.row + c.entry * r.q));
+  }
+  if (least / ctx->num_sms >= limit_us) return RBFFD_OK;
+  double us;
+  const TeamPlan T = plan_resident(mem, amg, ctx->num_sms, &us);
+  if (us >= limit_us) return RBFFD_OK;
+  const size_t bytes = krylov_res_args_bytes();
+  char *hb = (char *)S.hmem;
+  char *db = (char *)S.dmem;
+  unsigned int *dflags = (unsigned int *)(db + S.off_flags[slot]);
+  GridBarrier *dbars = (GridBarrier *)(db + S.off_bars[slot]);
+  for (int i = 0; i < m; ++i) {
+    int k = 0;
+    while (RES_SIZES[k] != T.nb[i]) ++k;
+    KrylovArgs a = at_size(args[i], probs[i], k);
+    a.flags = dflags + i;  // one arrival counter per system
+    a.bar = dbars + i;
+    // a member's second single system (symmetry lines) sums in the second
+    // half of the member's partials
+    const bool second = i > 0 && probs[i - 1] == probs[i];
+    a.res.part = (char *)probs[i]->res.part + (second ? RES_PART_BYTES / 2 : 0);
+    member_args(i, a, hb + S.off_sys[slot] + bytes * i, &need);
+    smem = std::max(smem, need);
+  }
+  RBFFD_TRY(put_tables(S, slot, T, m, bytes));
+  RBFFD_CK(cudaMemsetAsync(dflags, 0, sizeof(unsigned int) * m, ctx->stream));
+  RBFFD_TRY(reset_barriers(ctx, dbars, m));
+  *ran = true;
+  return krylov_res_batch_launch(ctx, nr, amg, T.nctas, db + S.off_sys[slot],
+                                 (const int *)(db + S.off_cta_sys[slot]),
+                                 (const int *)(db + S.off_cta_first[slot]), smem);
+}
+
 // One batched Krylov launch for the systems args[0..m) (args filled except
 // nblocks, tpr, flags and bar, which are set here), with table slot `slot`,
 // planned as a persistent work list from the systems' work (plan_teams).
 static int launch_krylov(BatchScratch &S, int slot, int nr, std::vector<KrylovArgs> &args,
                          const std::vector<double> &work, const std::vector<int> &rows,
-                         bool amg = false) {
+                         const std::vector<const rbffd_problem *> &probs, bool amg = false) {
   rbffd_ctx *ctx = S.ctx;
   const int m = (int)args.size();
   const int cmax = krylov_batch_max_ctas(ctx, nr);
@@ -411,9 +641,23 @@ static int launch_krylov(BatchScratch &S, int slot, int nr, std::vector<KrylovAr
   }
   std::vector<int> cap(m);
   for (int i = 0; i < m; ++i) cap[i] = args[i].nblocks;
-  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot]);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
+  double span;
+  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot], &span);
+  double all_rows = 0.0;
+  for (int i = 0; i < m; ++i) all_rows += i > 0 && probs[i] == probs[i - 1] ? 0.0 : rows[i];
+  if (S.scale[slot] == 1.0 && all_rows <= resident_rows(ctx)) {
+    double entries = 0.0, total = 0.0;
+    for (int i = 0; i < m; ++i) {
+      entries += work[i] * args[i].q;
+      total += work[i];
+    }
+    bool ran;
+    RBFFD_TRY(launch_resident(S, slot, nr, args, work, rows, probs, amg,
+                              STREAM_UNIT[amg] * entries / total * span, &ran));
+    if (ran) return RBFFD_OK;
+  }
   KrylovArgs *hsys = (KrylovArgs *)(hb + S.off_sys[slot]);
   unsigned int *dflags = (unsigned int *)(db + S.off_flags[slot]);
   GridBarrier *dbars = (GridBarrier *)(db + S.off_bars[slot]);
@@ -450,7 +694,8 @@ static int launch_mixed(BatchScratch &S, int slot, int nr, int inner,
   }
   std::vector<int> cap(m);
   for (int i = 0; i < m; ++i) cap[i] = args[i].nblocks;
-  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot]);
+  double span;
+  const TeamPlan T = plan_launch(work, cap, rows, cmax, S.scale[slot], &span);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
   MixedArgs *hsys = (MixedArgs *)(hb + S.off_sys[slot]);
@@ -484,8 +729,9 @@ static int launch_fgmres(BatchScratch &S, int slot, std::vector<FgmresArgs> &arg
     set_error("batch: %d members exceed the %d co-resident CTAs of one launch", m, cmax);
     return RBFFD_EINVAL;
   }
+  double span;
   const TeamPlan T =
-      plan_launch(work, std::vector<int>(m, kdev::MAXB), rows, cmax, S.scale[slot]);
+      plan_launch(work, std::vector<int>(m, kdev::MAXB), rows, cmax, S.scale[slot], &span);
   char *hb = (char *)S.hmem;
   char *db = (char *)S.dmem;
   FgmresArgs *hsys = (FgmresArgs *)(hb + S.off_sys[slot]);
@@ -520,6 +766,7 @@ static int launch_pcorr(BatchScratch &S, rbffd_problem *const *P, const std::vec
   std::vector<int> rj, ra, rf;
   std::vector<double> wj, wa, wf;
   std::vector<std::pair<int, int>> mj, ma, mf;
+  std::vector<const rbffd_problem *> qj, qa;
   for (size_t s = 0; s < sel.size(); ++s) {
     rbffd_problem *Q = P[sel[s]];
     if (Q->amgf) {
@@ -571,23 +818,25 @@ static int launch_pcorr(BatchScratch &S, rbffd_problem *const *P, const std::vec
       pa.push_back(a);
       ra.push_back(Q->n);
       wa.push_back(work_of(Q, 1));
+      qa.push_back(Q);
       ma.push_back({sel[s], 1});
     } else {
       pj.push_back(a);
       rj.push_back(Q->n);
       wj.push_back(work_of(Q, 1));
+      qj.push_back(Q);
       mj.push_back({sel[s], 1});
     }
   }
   if (!pj.empty()) {
     RBFFD_TRY(tune_mark(S, 2, 0));
-    RBFFD_TRY(launch_krylov(S, 2, 1, pj, wj, rj));
+    RBFFD_TRY(launch_krylov(S, 2, 1, pj, wj, rj, qj));
     S.slot_sys[2] = mj;
     RBFFD_TRY(tune_mark(S, 2, 1));
   }
   if (!pa.empty()) {
     RBFFD_TRY(tune_mark(S, 3, 0));
-    RBFFD_TRY(launch_krylov(S, 3, 1, pa, wa, ra, true));
+    RBFFD_TRY(launch_krylov(S, 3, 1, pa, wa, ra, qa, true));
     S.slot_sys[3] = ma;
     RBFFD_TRY(tune_mark(S, 3, 1));
   }
@@ -611,6 +860,7 @@ static int issue_batch(BatchScratch &S, rbffd_problem *const *P, int m,
   std::vector<KrylovArgs> a2, a1s;
   std::vector<int> rows2, rows1s;
   std::vector<double> work2, work1s;
+  std::vector<const rbffd_problem *> prob2, prob1s;
   std::vector<std::pair<int, int>> mem2, mem1s, xmem2[2], xmem1s[2];
   // mixed-precision members by inner arithmetic (0 FP32, 1 float-float)
   std::vector<MixedArgs> x2[2], x1s[2];
@@ -707,6 +957,7 @@ static int issue_batch(BatchScratch &S, rbffd_problem *const *P, int m,
       a2.push_back(a);
       rows2.push_back(P[i]->n);
       work2.push_back(work_of(P[i], 0));
+      prob2.push_back(P[i]);
       mem2.push_back({i, 0});
     } else {
       KrylovArgs au = a;
@@ -726,6 +977,8 @@ static int issue_batch(BatchScratch &S, rbffd_problem *const *P, int m,
       rows1s.push_back(P[i]->n);
       work1s.push_back(work_of(P[i], 0));
       work1s.push_back(work_of(P[i], 0));
+      prob1s.push_back(P[i]);
+      prob1s.push_back(P[i]);
       mem1s.push_back({i, 0});
       mem1s.push_back({i, 0});
     }
@@ -733,13 +986,13 @@ static int issue_batch(BatchScratch &S, rbffd_problem *const *P, int m,
   prof_begin(ctx, 0);
   if (!a2.empty()) {
     RBFFD_TRY(tune_mark(S, 0, 0));
-    RBFFD_TRY(launch_krylov(S, 0, 2, a2, work2, rows2));
+    RBFFD_TRY(launch_krylov(S, 0, 2, a2, work2, rows2, prob2));
     S.slot_sys[0] = mem2;
     RBFFD_TRY(tune_mark(S, 0, 1));
   }
   if (!a1s.empty()) {
     RBFFD_TRY(tune_mark(S, 1, 0));
-    RBFFD_TRY(launch_krylov(S, 1, 1, a1s, work1s, rows1s));
+    RBFFD_TRY(launch_krylov(S, 1, 1, a1s, work1s, rows1s, prob1s));
     S.slot_sys[1] = mem1s;
     RBFFD_TRY(tune_mark(S, 1, 1));
   }
@@ -891,6 +1144,14 @@ int batch_iterate(BatchScratch &S, rbffd_problem *const *P, int m,
   // hierarchies still being built are finished before anything is issued
   // (the iteration may be captured as a graph)
   for (int i = 0; i < m; ++i) RBFFD_TRY(amg_ready(P[i]));
+  // and what resident launches need of their members
+  double rows = 0.0;
+  for (int i = 0; i < m; ++i) rows += P[i]->precision == RBFFD_PREC_FP64 ? P[i]->n : 0.0;
+  if (rows > 0.0 && rows <= resident_rows(ctx)) {
+    RBFFD_TRY(team_sizes_ready(P, m));
+    for (int i = 0; i < m; ++i)
+      if (P[i]->precision == RBFFD_PREC_FP64) RBFFD_TRY(dense64_ready(P[i]));
+  }
   // a member with symmetry lines solves u~ and v~ as two single-RHS systems
   // (their rows differ there), so a launch may hold up to 2m systems
   RBFFD_TRY(S.reserve(ctx, 2 * m));

@@ -109,6 +109,14 @@ int krylov_launch(rbffd_ctx *ctx, int nr, int nblocks, const KrylovArgs &args);
 constexpr int RES_DENSE64_N = 512;  // most level-1 rows of an FP64 dense coarse operator
 int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgDev *h,
                       double omega, const double *B, bool *ran);
+// Batched: args.res holds the team (nb, R, hmax; hlist null: the kernel makes
+// the lists); the system's arguments (krylov_res_args_bytes) to out (null:
+// only whether it fits) and the shared memory its launch needs.
+size_t krylov_res_args_bytes();
+bool krylov_res_args(int nr, const KrylovArgs &args, const AmgDev *h, double omega,
+                     const double *B, void *out, size_t *smem);
+int krylov_res_batch_launch(rbffd_ctx *ctx, int nr, bool amg, int nctas, const void *d_sys,
+                            const int *d_cta_team, const int *d_info, size_t smem);
 int krylov_dense_ld(const AmgDev &h);
 int krylov_dense_build(rbffd_ctx *ctx, const AmgDev &h, double *B);
 size_t krylov_partials_doubles(int nr, int nblocks);

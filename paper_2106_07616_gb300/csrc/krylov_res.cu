@@ -20,7 +20,8 @@
 //
 // Measured on GB300, a whole FP64 outer iteration with the streaming and with
 // this solve: cavity 99^2 (q = 20, multigrid) 7.0 -> 4.1 ms, Kovasznay 30^2
-// (Jacobi, one cluster) 12.8 -> 4.8 ms.
+// (Jacobi, one cluster) 12.8 -> 4.8 ms; four requests of 5 184 to 8 836 rows
+// served together, two time steps each, batched: 500 -> 372 ms.
 #include "krylov.cuh"
 #include "resident.cuh"
 
@@ -60,6 +61,7 @@ struct BicgResArgs {
   // shared-memory layout, in bytes
   int o_val, o_idx, ld, o_list, o_w, o_vec, o_own, o_c1, o_b, o_rc, o_rv, o_pc, o_pv;
   int vres, bres, rcap, pcap;
+  int o_tmp;          // scratch of a halo list made by the kernel (batched launches)
 };
 
 __device__ __forceinline__ void ld_l2v(const res::Vec<double, 1> *p, res::Vec<double, 1> &v) {
@@ -71,8 +73,9 @@ __device__ __forceinline__ void ld_l2v(const res::Vec<double, 2> *p, res::Vec<do
   v.x[1] = t.y;
 }
 
+// The solve of one system by the nb CTAs of a team; this CTA is number lb.
 template <int NR, bool AMGP>
-__global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ BicgResArgs A) {
+__device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb, const int nb) {
   static_assert(!AMGP || NR == 1, "the multigrid preconditioner serves one right-hand side");
   using V = res::Vec<double, NR>;
   constexpr int VA = 3 * NR, VC = 5 * NR;
@@ -81,10 +84,10 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
   __shared__ int s_any;
   extern __shared__ __align__(16) unsigned char dyn[];
   const KrylovArgs &K = A.k;
-  const int lb = blockIdx.x, nb = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int s_len, s_own;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = K.n, q = K.q, ldn = K.ldn, T = A.T;
   const int R = K.res.R, r0 = min(n, lb * R), r1 = min(n, r0 + R), nr = r1 - r0;
-  const int L = K.res.hinfo[2 * lb], own = K.res.hinfo[2 * lb + 1];
   const int hm = K.res.hmax;
   res::Team team{K.flags, &K.bar->err, lb, nb, K.res.cluster, 0u};
   double *part = reinterpret_cast<double *>(K.res.part);
@@ -117,8 +120,20 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
   const int row = r0 + rl;
 
   // ---- load the CTA's share
+  const bool listed = K.res.hlist != nullptr;
+  if (listed) {
+    if (tid == 0) {
+      s_len = K.res.hinfo[2 * lb];
+      s_own = K.res.hinfo[2 * lb + 1];
+    }
+    __syncthreads();
+  } else {
+    res::halo_local(n, q, ldn, K.col, r0, r1, reinterpret_cast<unsigned int *>(dyn + A.o_tmp),
+                    list, idx, A.ld, &s_len, &s_own);
+  }
+  const int L = s_len, own = s_own;
   for (int e = tid; e < L; e += RES_NT) {
-    const int c = __ldg(K.res.hlist + (size_t)lb * K.res.hstride + e);
+    const int c = listed ? __ldg(K.res.hlist + (size_t)lb * K.res.hstride + e) : list[e];
     list[e] = c;
     if (AMGP) {
       const double dg = __ldg(K.val + c);  // a row's first entry is its diagonal
@@ -131,7 +146,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
     const int j = e / nr, i = e - j * nr;
     const size_t s = (size_t)j * ldn + r0 + i;
     if (A.vres) val[j * A.ld + i] = __ldg(K.val + s);
-    idx[j * A.ld + i] = __ldg(K.res.lidx + s);
+    if (listed) idx[j * A.ld + i] = __ldg(K.res.lidx + s);
   }
   int rs0 = 0, rs1 = 0, ps0 = 0, ps1 = 0, pa = 0, pe = 0;
   bool rres = false, pres = false;
@@ -688,6 +703,29 @@ __global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ 
   }
 }
 
+template <int NR, bool AMGP>
+__global__ void __launch_bounds__(RES_NT, 1) k_bicg_res(const __grid_constant__ BicgResArgs A) {
+  bicg_res_body<NR, AMGP>(A, blockIdx.x, gridDim.x);
+}
+
+// Batched: a persistent work list as in krylov.cu, teams of 1024-thread CTAs.
+template <int NR, bool AMGP>
+__global__ void __launch_bounds__(RES_NT, 1)
+    k_bicg_res_batch(const BicgResArgs *__restrict__ sys, const int *__restrict__ cta_team,
+                     const int *__restrict__ info) {
+  __shared__ BicgResArgs A;
+  const int t = cta_team[blockIdx.x];
+  const int c0 = info[4 * t], nc = info[4 * t + 1], j0 = info[4 * t + 2], j1 = info[4 * t + 3];
+  for (int j = j0; j < j1; ++j) {
+    __syncthreads();
+    const int *src = reinterpret_cast<const int *>(sys + info[j]);
+    for (int k = threadIdx.x; k < (int)(sizeof(A) / 4); k += RES_NT)
+      reinterpret_cast<int *>(&A)[k] = src[k];
+    __syncthreads();
+    bicg_res_body<NR, AMGP>(A, blockIdx.x - c0, nc);
+  }
+}
+
 int round16(size_t v) { return (int)((v + 15) / 16 * 16); }
 constexpr size_t SMEM_LIMIT = 200 * 1024;
 
@@ -715,7 +753,10 @@ bool layout(BicgResArgs &a, int nr, bool amg, size_t *smem) {
     const size_t coarse = a.B ? 0 : (size_t)(a.C.nc + R1);
     a.o_c1 = take(8 * (coarse > (size_t)a.n1 ? coarse : (size_t)a.n1));
   }
-  if (at > SMEM_LIMIT) return false;
+  // the list's scratch lies over what is loaded after it
+  a.o_tmp = (int)at;
+  const size_t tmp = p.hlist ? 0 : 8 * (size_t)((a.k.n + 31) / 32);
+  if (at + tmp > SMEM_LIMIT) return false;
   a.vres = at + 8 * (size_t)q * a.ld <= SMEM_LIMIT;
   if (a.vres) a.o_val = take(8 * (size_t)q * a.ld);
   if (amg) {
@@ -729,8 +770,42 @@ bool layout(BicgResArgs &a, int nr, bool amg, size_t *smem) {
     a.o_pv = take(8 * (size_t)a.pcap);
     a.o_pc = take(4 * (size_t)a.pcap);
   }
-  *smem = at;
+  *smem = at > (size_t)a.o_tmp + tmp ? at : (size_t)a.o_tmp + tmp;
   return true;
+}
+
+// The arguments and shared memory of a solve on the plan of args.res, or false.
+bool res_args(int nr, const KrylovArgs &args, const AmgDev *h, double omega, const double *B,
+              BicgResArgs *out, size_t *smem) {
+  const ResPlan &p = args.res;
+  const bool amg = args.amg != nullptr;
+  if (amg && (!h || h->nlev < 2 || (h->nlev > 2 && h->comp.nc < 1))) return false;
+  BicgResArgs &a = *out;
+  memset(&a, 0, sizeof(a));
+  a.k = args;
+  a.T = lanes(p.R);
+  // published vectors, up to two right-hand sides side by side: ph and s, sh
+  // and t of the first system are adjacent in the allocation
+  a.pubt[0] = args.w[0].ph;
+  a.pubv[0] = args.w[0].sh;
+  if (amg) {
+    a.omega = omega;
+    a.n1 = h->lev[1].n;
+    a.R0 = h->lev[0].R;
+    a.P0 = h->lev[0].P;
+    a.S1 = h->lev[1].S;
+    a.C = h->comp;
+    a.b1 = h->lev[1].b;
+    a.y1 = h->lev[1].y;
+    if (h->nlev == 2) {
+      a.B = h->cinv;
+      a.ldb = a.n1;
+    } else if (B) {
+      a.B = B;
+      a.ldb = a.n1;
+    }
+  }
+  return layout(a, nr, amg, smem);
 }
 
 // Row i of B = S_1 + sum_c Q(i, c) Rh(c, :), as in fgmres_res.cu.
@@ -774,34 +849,9 @@ int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgD
   const ResPlan &p = args.res;
   if (p.nb < 1 || p.hmax < 1 || p.hmax > p.hstride) return RBFFD_OK;
   const bool amg = args.amg != nullptr;
-  if (amg && (!h || h->nlev < 2 || (h->nlev > 2 && h->comp.nc < 1))) return RBFFD_OK;
   BicgResArgs a;
-  memset(&a, 0, sizeof(a));
-  a.k = args;
-  a.T = lanes(p.R);
-  // published vectors, up to two right-hand sides side by side: ph and s, sh
-  // and t of the first system are adjacent in the allocation
-  a.pubt[0] = args.w[0].ph;
-  a.pubv[0] = args.w[0].sh;
-  if (amg) {
-    a.omega = omega;
-    a.n1 = h->lev[1].n;
-    a.R0 = h->lev[0].R;
-    a.P0 = h->lev[0].P;
-    a.S1 = h->lev[1].S;
-    a.C = h->comp;
-    a.b1 = h->lev[1].b;
-    a.y1 = h->lev[1].y;
-    if (h->nlev == 2) {
-      a.B = h->cinv;
-      a.ldb = a.n1;
-    } else if (B) {
-      a.B = B;
-      a.ldb = a.n1;
-    }
-  }
   size_t smem = 0;
-  if (!layout(a, nr, amg, &smem)) return RBFFD_OK;
+  if (!res_args(nr, args, h, omega, B, &a, &smem)) return RBFFD_OK;
   RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
   if (!p.cluster) RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
   *ran = true;
@@ -809,6 +859,34 @@ int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgD
                    : nr == 1 ? (const void *)k_bicg_res<1, false>
                              : (const void *)k_bicg_res<2, false>;
   return res_launch(ctx, p, fn, &a, smem, "k_bicg_res");
+}
+
+size_t krylov_res_args_bytes() { return sizeof(BicgResArgs); }
+
+bool krylov_res_args(int nr, const KrylovArgs &args, const AmgDev *h, double omega,
+                     const double *B, void *out, size_t *smem) {
+  static_assert(sizeof(BicgResArgs) % 8 == 0, "copied as words");
+  BicgResArgs a;
+  if (!res_args(nr, args, h, omega, B, &a, smem)) return false;
+  if (out) memcpy(out, &a, sizeof(a));
+  return true;
+}
+
+int krylov_res_batch_launch(rbffd_ctx *ctx, int nr, bool amg, int nctas, const void *d_sys,
+                            const int *d_cta_team, const int *d_info, size_t smem) {
+  const void *fn = amg       ? (const void *)k_bicg_res_batch<1, true>
+                   : nr == 1 ? (const void *)k_bicg_res_batch<1, false>
+                             : (const void *)k_bicg_res_batch<2, false>;
+  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  void *kargs[] = {(void *)&d_sys, (void *)&d_cta_team, (void *)&d_info};
+  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nctas), dim3(RES_NT), kargs, smem,
+                                                    ctx->stream);
+  ctx->launches++;
+  if (e != cudaSuccess) {
+    set_error("cooperative launch of k_bicg_res_batch failed: %s", cudaGetErrorString(e));
+    return RBFFD_ECUDA;
+  }
+  return RBFFD_OK;
 }
 
 }  // namespace rbffd

@@ -222,6 +222,8 @@ int build(rbffd_problem *P, const rbffd_problem_desc *d) {
   RBFFD_CK(cudaStreamSynchronize(st));
   const int hfs = back[0];
   P->res.hmax = back[1];
+  P->res_hm_known = false;
+  memset(P->res_hm, 0, sizeof(P->res_hm));
   if (ctx->prof) {
     const double N = P->q + (P->degree + 1) * (P->degree + 2) / 2;
     const double flops = 2.0 * N * N * N / 3.0 + 6.0 * N * N + 10.0 * P->q * P->q;
@@ -385,14 +387,7 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
   a.w[1] = P->kv[1];
   a.out = P->kout + 2;
   a.tpr = krylov_threads_per_row(P->n, 1, P->kblocks1);
-  if (a.amg) {
-    const int ld = P->res.nb > 0 && !P->amgB ? krylov_dense_ld(P->amg_host) : 0;
-    const size_t bytes = sizeof(double) * (size_t)ld * ld;
-    if (ld > 0 && dev_alloc(ctx, (void **)&P->amgB, bytes) == RBFFD_OK) {
-      P->fgB_bytes = bytes;
-      RBFFD_TRY(krylov_dense_build(ctx, P->amg_host, P->amgB));
-    }
-  }
+  if (a.amg) RBFFD_TRY(dense64_ready(P));
   return issue_fp64(P, 1, P->kblocks1, a);
 }
 
@@ -601,6 +596,33 @@ int rbffd::compat_fallback(rbffd_problem *P, double *relres) {
   return rc;
 }
 
+int rbffd::team_sizes_ready(rbffd_problem *const *P, int m) {
+  bool any = false;
+  for (int i = 0; i < m; ++i) {
+    rbffd_problem *Q = P[i];
+    if (Q->res_hm_known || Q->res.nb == 0) continue;
+    int *d_hm = Q->d_first_singular + 2;
+    RBFFD_TRY(res_halo_sizes(Q->ctx, Q->n, Q->q, Q->ldn, Q->col, d_hm));
+    RBFFD_CK(cudaMemcpyAsync(Q->res_hm, d_hm, sizeof(Q->res_hm), cudaMemcpyDeviceToHost,
+                             Q->ctx->stream));
+    any = true;
+  }
+  if (!any) return RBFFD_OK;
+  RBFFD_CK(cudaStreamSynchronize(P[0]->ctx->stream));
+  for (int i = 0; i < m; ++i) P[i]->res_hm_known = true;
+  return RBFFD_OK;
+}
+
+int rbffd::dense64_ready(rbffd_problem *P) {
+  const int ld = P->amg && P->res.nb > 0 && !P->amgB ? krylov_dense_ld(P->amg_host) : 0;
+  const size_t bytes = sizeof(double) * (size_t)ld * ld;
+  if (ld > 0 && dev_alloc(P->ctx, (void **)&P->amgB, bytes) == RBFFD_OK) {
+    P->fgB_bytes = bytes;
+    RBFFD_TRY(krylov_dense_build(P->ctx, P->amg_host, P->amgB));
+  }
+  return RBFFD_OK;
+}
+
 int rbffd::compat_ready(rbffd_problem *P) {
   if (!P->compat || P->z_ready) return RBFFD_OK;
   RBFFD_TRY(amg_ready(P));
@@ -680,7 +702,7 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
     size_t o_bar = c.take<GridBarrier>(1);
     size_t o_flags = c.take<unsigned int>(256);
     size_t o_rec = c.take<Readback>(1);
-    size_t o_fs = c.take<int>(2);
+    size_t o_fs = c.take<int>(2 + RES_NSIZES);
     size_t o_knn = c.take<char>(P->knn_lay.bytes);
     size_t o_p32 = 0, o_a32 = 0, o_pd32 = 0, o_md32 = 0, o_mv[18] = {}, o_part64 = 0, o_part32 = 0;
     size_t o_a32b = 0, o_md32b = 0;

@@ -53,6 +53,9 @@ struct rbffd_problem {
   rbffd::ResPlan res;
   int32_t *res_hlist = nullptr, *res_hinfo = nullptr;
   uint16_t *res_lidx = nullptr;
+  // longest halo list at each team size of a batched resident solve (0: none)
+  int res_hm[rbffd::RES_NSIZES] = {};
+  bool res_hm_known = false;
   // fields
   double *u, *v, *p, *p2, *un, *vn, *unm1, *vnm1, *ut, *vt, *pc, *bu, *bv, *bp;
   // compatible p' of a pinned problem (no outlet): z = M^{-1} e_I, solved
@@ -129,6 +132,11 @@ bool steady_done(const rbffd_solve_params *s, double R, double change, int steps
 // on the problem's stream); a no-op when none is pending.  Every use of
 // the hierarchy calls it first.
 int amg_ready(rbffd_problem *P);
+// res_hm of every member (one wait for the host; before any capture).
+int team_sizes_ready(rbffd_problem *const *P, int m);
+// The FP64 resident p' solve's dense coarse operator, made once per hierarchy
+// (amg_ready first; without memory for it the solves run without).
+int dense64_ready(rbffd_problem *P);
 // Solve z = M^{-1} e_I with the problem's p' solver once per build (pinned
 // problems only; a no-op otherwise or when done).  Synchronises the stream:
 // call it before any graph capture.

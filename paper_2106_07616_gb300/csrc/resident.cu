@@ -76,7 +76,42 @@ __global__ void __launch_bounds__(RES_NT) k_halo_build(int n, int q, int ldn, in
   }
 }
 
+// The longest list at each team size: CTA b is CTA b - first of size k's team.
+struct SizeTable {
+  int nb[RES_NSIZES], first[RES_NSIZES + 1];
+};
+__global__ void __launch_bounds__(RES_NT) k_halo_sizes(int n, int q, int ldn, SizeTable t,
+                                                       const int32_t *__restrict__ col,
+                                                       int *hm) {
+  extern __shared__ unsigned int bm[];
+  __shared__ int len, own;
+  int k = 0;
+  while (blockIdx.x >= t.first[k + 1]) ++k;
+  const int R = (n + t.nb[k] - 1) / t.nb[k], b = blockIdx.x - t.first[k];
+  const int r0 = min(n, b * R), r1 = min(n, r0 + R);
+  res::halo_local(n, q, ldn, col, r0, r1, bm, nullptr, nullptr, 0, &len, &own);
+  if (threadIdx.x == 0) atomicMax(hm + k, len);
+}
+
 }  // namespace
+
+int res_halo_sizes(rbffd_ctx *ctx, int n, int q, int ldn, const int32_t *col, int *d_hm) {
+  SizeTable t;
+  int at = 0;
+  for (int k = 0; k < RES_NSIZES; ++k) {
+    t.first[k] = at;
+    const int nb = t.nb[k] = RES_SIZES[k];
+    if ((long long)nb * RES_NT >= n && nb <= ctx->num_sms) at += nb;
+  }
+  t.first[RES_NSIZES] = at;
+  RBFFD_CK(cudaMemsetAsync(d_hm, 0, sizeof(int) * RES_NSIZES, ctx->stream));
+  if (at == 0) return RBFFD_OK;
+  const size_t smem = 2 * sizeof(unsigned int) * (size_t)((n + 31) / 32);
+  RBFFD_CK(cudaFuncSetAttribute(k_halo_sizes, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(2 * sizeof(unsigned int) * ((RES_MAXN + 31) / 32))));
+  k_halo_sizes<<<at, RES_NT, smem, ctx->stream>>>(n, q, ldn, t, col, d_hm);
+  return after_launch(ctx, "k_halo_sizes");
+}
 
 ResPlan res_plan(rbffd_ctx *ctx, int n) {
   ResPlan p;

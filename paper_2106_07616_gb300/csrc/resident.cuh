@@ -47,6 +47,13 @@ struct ResPlan {
 // partial sums of a grid team: two halves of up to 64 values of 8 bytes
 constexpr size_t RES_PART_BYTES = 2 * 64 * RES_MAXB * 8;
 
+// Team sizes a batched resident launch chooses from, and for a problem the
+// longest halo list at each (0: the team would not fit its rows).
+constexpr int RES_NSIZES = 15;
+constexpr int RES_SIZES[RES_NSIZES] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 152};
+// Longest lists of the sizes that suit n rows to d_hm[RES_NSIZES] (device).
+int res_halo_sizes(rbffd_ctx *ctx, int n, int q, int ldn, const int32_t *col, int *d_hm);
+
 // Rows and lanes of a team for n rows (nb = 0 when a CTA would own more rows
 // than it has threads).
 ResPlan res_plan(rbffd_ctx *ctx, int n);
@@ -224,6 +231,71 @@ __device__ __forceinline__ bool team_totals(Team &t, P (&val)[pow2_ge(V)], P *to
     __syncthreads();
   }
   return ok;
+}
+
+// The halo list of the CTA's rows [r0, r1) made by the CTA itself (a batched
+// launch chooses its teams after the build): the sorted columns to list (n2
+// at most), every entry's place to idx[j * ld + row].  bm: 2 ceil(n / 32)
+// words of shared scratch.  The length and the place of the first row to
+// *len and *own (shared).  Ends with a barrier.
+__device__ __forceinline__ void halo_local(int n, int q, int ldn, const int32_t *__restrict__ col,
+                                           int r0, int r1, unsigned int *bm, int *list,
+                                           uint16_t *idx, int ld, int *len, int *own) {
+  __shared__ unsigned int wtot[RES_NT / 32];
+  const int W = (n + 31) / 32, nr = r1 - r0;
+  unsigned int *pre = bm + W;
+  for (int k = threadIdx.x; k < W; k += RES_NT) bm[k] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < nr * q; e += RES_NT) {
+    const int j = e / nr, i = r0 + e - j * nr;
+    const int c = __ldg(col + (size_t)j * ldn + i);
+    atomicOr(bm + (c >> 5), 1u << (c & 31));
+  }
+  __syncthreads();
+  // exclusive scan of the words' counts: a run of words per thread, then
+  // warps, then the block
+  const int cw = (W + RES_NT - 1) / RES_NT, k0 = min(W, (int)threadIdx.x * cw),
+            k1 = min(W, k0 + cw);
+  unsigned int mine = 0;
+  for (int k = k0; k < k1; ++k) mine += __popc(bm[k]);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned int inc = mine;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) wtot[w] = inc;
+  __syncthreads();
+  unsigned int base = 0, total = 0;
+  for (int k = 0; k < RES_NT / 32; ++k) {
+    if (k < w) base += wtot[k];
+    total += wtot[k];
+  }
+  unsigned int at = base + inc - mine;
+  for (int k = k0; k < k1; ++k) {
+    pre[k] = at;
+    unsigned int bits = bm[k];
+    while (bits) {
+      const int o = __ffs(bits) - 1;
+      bits &= bits - 1;
+      if (list != nullptr) list[at] = 32 * k + o;
+      ++at;
+    }
+  }
+  __syncthreads();
+  auto place = [&](int c) {
+    return pre[c >> 5] + __popc(bm[c >> 5] & ((1u << (c & 31)) - 1u));
+  };
+  if (idx != nullptr)
+    for (int e = threadIdx.x; e < nr * q; e += RES_NT) {
+      const int j = e / nr, i = e - j * nr;
+      idx[j * ld + i] = (uint16_t)place(__ldg(col + (size_t)j * ldn + r0 + i));
+    }
+  if (threadIdx.x == 0) {
+    *len = (int)total;
+    *own = nr > 0 ? (int)place(r0) : 0;
+  }
+  __syncthreads();
 }
 
 // ---- values of NR right-hand sides side by side -----------------------------

@@ -76,3 +76,36 @@ def test_resident_fgmres_on_outlet_channels(case):
         assert rel_l2(P.get(k), Q.get(k)) <= 1e-6, k
     P.close()
     Q.close()
+
+
+BATCHES = {
+    "pair": ("two_ctas", "grid_least"),
+    "every": tuple(sorted(CASES)),
+    # more systems than teams: a team takes several in turn
+    "many": ("one_cta", "two_ctas", "symmetry") * 60,
+}
+
+
+@pytest.mark.parametrize("precond", [rbffd.PRECOND_JACOBI, rbffd.PRECOND_AMG])
+@pytest.mark.parametrize("name", sorted(BATCHES))
+def test_resident_batch_matches_oracle(name, precond):
+    """The batched launches' teams: halo lists made by the kernel, sizes out of
+    a table, single right-hand sides in pairs; tolerances as above."""
+    fps = {c: CASES[c]() for c in BATCHES[name]}
+    probs = [rbffd.Problem(ctx(), fps[c], rbffd.PREC_FP64, precond=precond)
+             for c in BATCHES[name]]
+    B = rbffd.Batch(ctx(), probs)
+    _, _, status = B.iterate([fps[c].dt for c in BATCHES[name]], krylov_tol=1e-12,
+                             krylov_maxit=100000)
+    assert not status.any()
+    want = {}
+    for c, P in zip(BATCHES[name], probs):
+        if c not in want:
+            O = oracle.Problem(fps[c], krylov_tol=1e-12, krylov_maxit=100000)
+            O.simple_iterate(fps[c].dt)
+            want[c] = O
+        for k in FIELDS:
+            assert rel_l2(P.get(k), want[c].get(k)) <= 1e-8, (c, k)
+    B.close()
+    for P in probs:
+        P.close()
