@@ -1,4 +1,4 @@
-// weights.cu -- S2: PHS r^3 + polynomial collocation weights, one warp per
+// weights.cu -- S2: PHS r^3 + polynomial collocation weights, 4 to 32 lanes a
 // cloud, the augmented (q+m) x (q+m+3) system in shared memory, FP64 LU with
 // partial pivoting (paper Sec. 2, Eqs. RBF_interp_mat_vec ..
 // RBF_interp_mat_vec_L_solve).
@@ -11,84 +11,56 @@
 //   - the system is eliminated through the null space of the polynomials
 //     (k_weights), 32 k flops a cloud instead of 73 k at q = 30, m = 15;
 //   - updates are one fused multiply-add, dealt element by element over the
-//     32 lanes, so every FP64 instruction of the warp carries 32 of them;
+//     cloud's lanes, so every FP64 instruction of the warp carries 32 of them;
 //   - one reciprocal per pivot, kept for the back substitution (a division is
-//     a sequence of FP64 instructions whatever its active lanes);
+//     a sequence of FP64 instructions whatever its active lanes), and small
+//     clouds several to a warp, which then share it;
+//   - a monomial is one product of two powers that are there;
 //   - Phi is symmetric: each r^3 (and its square root) is computed once for
 //     the upper triangle and stored twice; S = Z^T Phi Z likewise.
 // The weights then differ from the oracle's elimination of the whole matrix
 // by rounding only, well inside the 1e-10 they are held to.  Measured on
 // GB300: 40 000 clouds at q = 30, degree 4 in 5.8 ms by elimination of the
-// augmented matrix, 3.2 ms this way (error against 64-bit LAPACK 8e-14 and
-// 1.3e-13 relative); 10 201 clouds at q = 12, degree 2 in 0.47 and 0.25 ms.
+// augmented matrix, 3.2 ms by the null space with a warp a cloud and 16 warps a
+// block, 2.4 ms now: some 1 200 FP64 instructions a cloud, 19 000 cycles, keep
+// the pipe busy (error against 64-bit LAPACK 8e-14 and 1.3e-13 relative);
+// 10 201 clouds at q = 12, degree 2 in 0.47, 0.25 and 0.11 ms.
 #include "abi_guard.cuh"
 #include "common.cuh"
 #include "weights.cuh"
 
 namespace rbffd {
 
-// Monomial exponents in graded order, x power descending inside a degree:
-// 1, x, y, x^2, xy, y^2, ...  The order for degree k is a prefix of the
-// order for degree k+1, so one table serves every degree up to 8.
-__constant__ int8_t c_ax[45];
-__constant__ int8_t c_ay[45];
-
-static bool g_tables_ready[64] = {false};
-
-static int ensure_tables(int device) {
-  if (device >= 0 && device < 64 && g_tables_ready[device]) return RBFFD_OK;
-  int8_t ax[45], ay[45];
-  int l = 0;
-  for (int d = 0; d <= 8; ++d)
-    for (int a = d; a >= 0; --a) {
-      ax[l] = (int8_t)a;
-      ay[l] = (int8_t)(d - a);
-      ++l;
-    }
-  RBFFD_CK(cudaMemcpyToSymbol(c_ax, ax, sizeof(ax)));
-  RBFFD_CK(cudaMemcpyToSymbol(c_ay, ay, sizeof(ay)));
-  if (device >= 0 && device < 64) g_tables_ready[device] = true;
-  return RBFFD_OK;
-}
-
-// A warp's shared memory, in doubles (odd leading dimensions: column walks
+// A cloud's shared memory, in doubles (odd leading dimensions: column walks
 // touch every bank).
 struct WeightsLayout {
-  int ldp, ldf, f, xi, rhs, g, inv, ord, total;
+  int ldp, ldf, f, xi, ord, total;
   __host__ __device__ WeightsLayout(int q, int m) {
     ldp = m | 1;
-    ldf = q | 1;
-    f = q * ldp;
+    ldf = (q + 3) | 1;
+    f = (q + 3) * ldp;
     xi = f + q * ldf;
-    rhs = xi + 2 * q;
-    g = rhs + 3 * q;
-    inv = g + 3 * m;
-    ord = inv + m;
+    ord = xi + 2 * q;
     total = ord + (q + 1) / 2;
   }
 };
 
-__device__ __forceinline__ double ipow_rn(double b, int e) {
-  double v = 1.0;
-  for (int t = 0; t < e; ++t) v = __dmul_rn(v, b);
-  return v;
-}
-
-// Largest |v[e * ld]| of e = k .. n - 1 over the warp, on bit patterns: for
+// Largest |v[e * ld]| of e = k .. n - 1 over the cloud's LW lanes, on bit patterns: for
 // finite doubles with the sign bit cleared, unsigned 64-bit order is the
 // order of the values, so this picks exactly the row an FP64 comparison would
 // (ties to the lowest row) while keeping the compares off the FP64 pipe.
 // Returns the row, or n if every entry is zero.
+template <int LW>
 __device__ __forceinline__ int pivot_row(const double *v, int ld, int k, int n, int lane) {
   unsigned long long best = 0ull;
   int piv = n;
-  for (int r = k + lane; r < n; r += 32) {
+  for (int r = k + lane; r < n; r += LW) {
     const unsigned long long a =
         (unsigned long long)__double_as_longlong(v[r * ld]) & 0x7fffffffffffffffull;
     if (a > best) { best = a; piv = r; }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = LW / 2; o > 0; o >>= 1) {
     const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
     const int op = __shfl_xor_sync(0xffffffffu, piv, o);
     if (ob > best || (ob == best && op < piv)) { best = ob; piv = op; }
@@ -105,6 +77,7 @@ __device__ __forceinline__ double ratio(double a, double pivot, double inv) {
 // Rank-one update of rows r0 .. nr - 1, columns c0 .. nc - 1 of M by column k
 // and row k, the elements dealt over the lanes in row-major order so that
 // every FP64 instruction of the warp carries 32 updates.
+template <int LW>
 __device__ __forceinline__ void rank_one(double *M, int ld, int k, int r0, int nr, int c0, int nc,
                                          int lane) {
   const int C = nc - c0, E = (nr - r0) * C;
@@ -112,306 +85,282 @@ __device__ __forceinline__ void rank_one(double *M, int ld, int k, int r0, int n
   int r = r0 + lane / C, c = c0 + lane % C;
   int e = lane;
   // two elements per trip: their loads go out before either update
-  for (; e + 32 < E; e += 64) {
-    int r2 = r, c2 = c + 32;
+  for (; e + LW < E; e += 2 * LW) {
+    int r2 = r, c2 = c + LW;
     while (c2 >= nc) { c2 -= C; ++r2; }
     const double l1 = M[r * ld + k], u1 = M[k * ld + c], a1 = M[r * ld + c];
     const double l2 = M[r2 * ld + k], u2 = M[k * ld + c2], a2 = M[r2 * ld + c2];
     M[r * ld + c] = __fma_rn(-l1, u1, a1);
     M[r2 * ld + c2] = __fma_rn(-l2, u2, a2);
     r = r2;
-    c = c2 + 32;
+    c = c2 + LW;
     while (c >= nc) { c -= C; ++r; }
   }
   if (e < E) M[r * ld + c] = __fma_rn(-M[r * ld + k], M[k * ld + c], M[r * ld + c]);
 }
 
-// The weights of one cloud per warp by the null space of the polynomials.
+// The weights of one cloud per LW lanes by the null space of the polynomials.
 // The system [Phi P; P^T 0] [c; d] = [f; g] is eliminated in blocks:
 //   P = [L1; L2] U with partial pivoting (rows permuted, the cloud's points
 //     with them), K = L2 L1^-1, so Z = [-K^T; I] spans the null space of P^T;
-//   c = [L1^-T U^-T g; 0] + Z c2 meets the constraints for every c2;
-//   (Z^T Phi Z) c2 = Z^T (f - Phi c_p) by LU with partial pivoting, order
-//     q - m instead of q + m.
+//   c = [c_p; 0] + Z c2 with c_p = L1^-T U^-T g meets the constraints for
+//     every c2;
+//   (Z^T Phi Z) c2 = Z^T (f - Phi [c_p; 0]) by LU with partial pivoting,
+//     order q - m instead of q + m.
+// The right-hand sides ride along: g^T as three more rows of P (which become
+// c_p^T by the steps that make K), f as three more columns of Phi.
 // At q = 2 m this takes 32 k flops for q = 30 instead of 73 k (two thirds of
 // (q + m)^3 and the right-hand sides).  A cloud is singular when either
 // factorisation meets an exactly zero pivot, as the augmented matrix is.
-__global__ void k_weights(int n, const double *__restrict__ x, const double *__restrict__ y,
-                          int q, const int32_t *__restrict__ idx, int m, int wpb,
-                          double *__restrict__ wx, double *__restrict__ wy,
-                          double *__restrict__ wl, int *first_singular, double Lx, double Ly) {
+// Lanes a cloud: a warp's clouds share the instructions that one lane would
+// do for all (reciprocals) and the part-filled last ones of every loop.
+template <int LW>
+__global__ void __launch_bounds__(32)
+    k_weights(int n, const double *__restrict__ x, const double *__restrict__ y, int q,
+              const int32_t *__restrict__ idx, int m, int degree, double *__restrict__ wx,
+              double *__restrict__ wy, double *__restrict__ wl, int *first_singular, double Lx,
+              double Ly) {
   extern __shared__ double smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sub = threadIdx.x / LW, lane = threadIdx.x % LW;
   const WeightsLayout ly(q, m);
-  double *P = smem + (size_t)warp * ly.total;  // q x ldp: P, then L1 \ U over K
-  double *F = P + ly.f;                        // Phi, q x ldf
+  double *P = smem + (size_t)sub * ly.total;  // (q + 3) x ldp: P, then L1 \ U over K, c_p^T
+  double *F = P + ly.f;                       // q x ldf: Phi, then the right-hand sides
   double *xi = P + ly.xi, *eta = xi + q;
-  double *f = P + ly.rhs;                      // q x 3: right-hand sides, then c
-  double *g = P + ly.g;                        // m x 3: constraints, then c_p
-  double *inv = P + ly.inv;                    // m reciprocal pivots of P
   int *ord = reinterpret_cast<int *>(P + ly.ord);
   const int ldp = ly.ldp, ldf = ly.ldf, n2 = q - m;
-  for (int i = blockIdx.x * wpb + warp; i < n; i += gridDim.x * wpb) {
-    const int32_t *cl = idx + (int64_t)i * q;
-    const double xc = x[i], yc = y[i];
-    // cloud radius h = max distance
-    double d2m = 0.0;
-    for (int a = lane; a < q; a += 32) {
-      int j = cl[a];
-      double dx = pdiff(x[j], xc, Lx), dy = pdiff(y[j], yc, Ly);
-      double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-      d2m = fmax(d2m, d2);
-    }
+  // the warp's lanes stay together: past the last cloud they repeat it and
+  // write nothing
+  const int i0 = blockIdx.x * (32 / LW);
+  const bool out = i0 + sub < n;
+  const int i = out ? i0 + sub : n - 1;
+  const int32_t *cl = idx + (int64_t)i * q;
+  const double xc = x[i], yc = y[i];
+  // cloud radius h = max distance
+  double d2m = 0.0;
+  for (int a = lane; a < q; a += LW) {
+    int j = cl[a];
+    double dx = pdiff(x[j], xc, Lx), dy = pdiff(y[j], yc, Ly);
+    double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+    d2m = fmax(d2m, d2);
+  }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d2m = fmax(d2m, __shfl_xor_sync(0xffffffffu, d2m, o));
-    double h = __dsqrt_rn(d2m);
-    if (h == 0.0) h = 1.0;
-    const double hinv = __drcp_rn(h);
-    for (int a = lane; a < q; a += 32) {
-      int j = cl[a];
-      xi[a] = __dmul_rn(pdiff(x[j], xc, Lx), hinv);
-      eta[a] = __dmul_rn(pdiff(y[j], yc, Ly), hinv);
-      ord[a] = a;
+  for (int o = LW / 2; o > 0; o >>= 1) d2m = fmax(d2m, __shfl_xor_sync(0xffffffffu, d2m, o));
+  double h = __dsqrt_rn(d2m);
+  if (h == 0.0) h = 1.0;
+  const double hinv = __drcp_rn(h);
+  for (int a = lane; a < q; a += LW) {
+    int j = cl[a];
+    const double xa = __dmul_rn(pdiff(x[j], xc, Lx), hinv),
+                 ya = __dmul_rn(pdiff(y[j], yc, Ly), hinv);
+    xi[a] = xa;
+    eta[a] = ya;
+    ord[a] = a;
+    // monomials in graded order: degree d starts at d (d + 1) / 2 with x^d
+    // and ends with y^d; those between from the powers
+    double *p = P + a * ldp;
+    double px = 1.0, py = 1.0;
+    p[0] = 1.0;
+    for (int d = 1; d <= degree; ++d) {
+      px = __dmul_rn(px, xa);
+      py = __dmul_rn(py, ya);
+      double *pd = p + d * (d + 1) / 2;
+      pd[0] = px;
+      pd[d] = py;
+      for (int b = 1; b < d; ++b)  // x^(d-b) y^b
+        pd[b] = __dmul_rn(p[(d - b) * (d - b + 1) / 2], p[b * (b + 1) / 2 + b]);
+    }
+  }
+  // the operators of the monomials at the centre: d/dx of x, d/dy of y, the
+  // Laplacian of x^2 and y^2
+  for (int e = lane; e < 3 * m; e += LW) {
+    const int s = e / m, l = e - s * m;
+    P[(q + s) * ldp + l] = s < 2 ? (l == s + 1 ? 1.0 : 0.0) : l == 3 || l == 5 ? 2.0 : 0.0;
+  }
+  __syncwarp();
+  // ---- P = [L1; L2] U
+  bool singular = false;
+  for (int k = 0; k < m; ++k) {
+    int piv = pivot_row<LW>(P + k, ldp, k, q, lane);
+    if (piv >= q) { singular = true; piv = k; }
+    if (piv != k) {
+      for (int c = lane; c < m; c += LW) {
+        const double t = P[k * ldp + c];
+        P[k * ldp + c] = P[piv * ldp + c];
+        P[piv * ldp + c] = t;
+      }
+      if (lane == 0) {
+        const double tx = xi[k], ty = eta[k];
+        const int to = ord[k];
+        xi[k] = xi[piv];
+        eta[k] = eta[piv];
+        ord[k] = ord[piv];
+        xi[piv] = tx;
+        eta[piv] = ty;
+        ord[piv] = to;
+      }
     }
     __syncwarp();
-    for (int e = lane; e < q * m; e += 32) {
-      const int a = e / m, l = e - a * m;
-      P[a * ldp + l] = __dmul_rn(ipow_rn(xi[a], c_ax[l]), ipow_rn(eta[a], c_ay[l]));
-    }
-    // the operators of the monomials at the centre
-    for (int l = lane; l < m; l += 32) {
-      const int ax = c_ax[l], ay = c_ay[l];
-      g[3 * l] = (ax == 1 && ay == 0) ? 1.0 : 0.0;
-      g[3 * l + 1] = (ax == 0 && ay == 1) ? 1.0 : 0.0;
-      g[3 * l + 2] = ((ax == 2 && ay == 0) || (ax == 0 && ay == 2)) ? 2.0 : 0.0;
-    }
+    const double pk = P[k * ldp + k], kinv = __drcp_rn(pk);
+    for (int r = k + 1 + lane; r < q + 3; r += LW)
+      P[r * ldp + k] = ratio(P[r * ldp + k], pk, kinv);
     __syncwarp();
-    // ---- P = [L1; L2] U
-    bool singular = false;
-    for (int k = 0; k < m; ++k) {
-      const int piv = pivot_row(P + k, ldp, k, q, lane);
-      if (piv >= q) { singular = true; break; }
-      if (piv != k) {
-        for (int c = lane; c < m; c += 32) {
-          const double t = P[k * ldp + c];
-          P[k * ldp + c] = P[piv * ldp + c];
-          P[piv * ldp + c] = t;
-        }
-        if (lane == 0) {
-          const double tx = xi[k], ty = eta[k];
-          const int to = ord[k];
-          xi[k] = xi[piv];
-          eta[k] = eta[piv];
-          ord[k] = ord[piv];
-          xi[piv] = tx;
-          eta[piv] = ty;
-          ord[piv] = to;
-        }
-        __syncwarp();
-      }
-      const double pk = P[k * ldp + k], kinv = __drcp_rn(pk);
-      if (lane == 0) inv[k] = kinv;
-      for (int r = k + 1 + lane; r < q; r += 32)
-        P[r * ldp + k] = ratio(P[r * ldp + k], pk, kinv);
-      __syncwarp();
-      rank_one(P, ldp, k, k + 1, q, k + 1, m, lane);
-      __syncwarp();
-    }
-    if (!singular) {
-      // ---- K = L2 L1^-1 in place, a column at a time from the last
-      for (int j = m - 1; j > 0; --j) {
-        for (int e = lane; e < n2 * j; e += 32) {
-          const int r = m + e / j, c = e - (e / j) * j;
-          P[r * ldp + c] = __fma_rn(-P[r * ldp + j], P[j * ldp + c], P[r * ldp + c]);
-        }
-        __syncwarp();
-      }
-      // ---- c_p = L1^-T U^-T g
-      for (int j = 0; j < m; ++j) {
-        if (lane < 3) g[3 * j + lane] = __dmul_rn(g[3 * j + lane], inv[j]);
-        __syncwarp();
-        for (int e = lane; e < 3 * (m - 1 - j); e += 32) {
-          const int r = j + 1 + e / 3, s = e % 3;
-          g[3 * r + s] = __fma_rn(-P[j * ldp + r], g[3 * j + s], g[3 * r + s]);
-        }
-        __syncwarp();
-      }
-      for (int j = m - 1; j > 0; --j) {
-        for (int e = lane; e < 3 * j; e += 32) {
-          const int r = e / 3, s = e % 3;
-          g[3 * r + s] = __fma_rn(-P[j * ldp + r], g[3 * j + s], g[3 * r + s]);
-        }
-        __syncwarp();
-      }
-      // ---- Phi: r^3 of the permuted points, symmetric with a zero diagonal;
-      // the q(q-1)/2 pairs a < b dealt over the lanes in row-major order
-      for (int a = lane; a < q; a += 32) F[a * ldf + a] = 0.0;
-      {
-        // pair number e -> (a, b): past the end of row a (b >= q) it goes on
-        // at b - q positions into row a + 1, whose first pair is (a+1, a+2)
-        const int np = q * (q - 1) / 2;
-        int a = 0, b = 1 + lane;
-        while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
-        for (int e = lane; e < np; e += 32) {
-          const double dx = __dsub_rn(xi[a], xi[b]), dy = __dsub_rn(eta[a], eta[b]);
-          const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-          const double r3 = __dmul_rn(__dsqrt_rn(d2), d2);
-          F[a * ldf + b] = r3;
-          F[b * ldf + a] = r3;
-          b += 32;
-          while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
-        }
-      }
-      // right-hand sides: d/dxi, d/deta and Laplacian of r^3 about the centre
-      for (int a = lane; a < q; a += 32) {
-        const double xa = xi[a], ya = eta[a];
-        const double rj = __dsqrt_rn(__dadd_rn(__dmul_rn(xa, xa), __dmul_rn(ya, ya)));
-        const double r3 = __dmul_rn(3.0, rj);
-        f[3 * a] = __dmul_rn(r3, __dsub_rn(0.0, xa));
-        f[3 * a + 1] = __dmul_rn(r3, __dsub_rn(0.0, ya));
-        f[3 * a + 2] = __dmul_rn(9.0, rj);
-      }
-      __syncwarp();
-      // f -= Phi c_p (before Phi12 is overwritten)
-      for (int e = lane; e < 3 * q; e += 32) {
-        const int a = e / 3, s = e % 3;
-        double t = f[e];
-        for (int l = 0; l < m; ++l) t = __fma_rn(-F[a * ldf + l], g[3 * l + s], t);
-        f[e] = t;
-      }
-      __syncwarp();
-      // M = Phi12 - Phi11 K^T over Phi12; f2 -= K f1
-      for (int e = lane; e < m * n2; e += 32) {
-        const int a = e / n2, b = e - a * n2;
-        const double *ka = P + (m + b) * ldp, *fa = F + a * ldf;
-        double t = fa[m + b];
-        for (int l = 0; l < m; ++l) t = __fma_rn(-fa[l], ka[l], t);
-        F[a * ldf + m + b] = t;
-      }
-      for (int e = lane; e < 3 * n2; e += 32) {
-        const int b = e / 3, s = e % 3;
-        double t = f[3 * m + e];
-        for (int l = 0; l < m; ++l) t = __fma_rn(-P[(m + b) * ldp + l], f[3 * l + s], t);
-        f[3 * m + e] = t;
-      }
-      __syncwarp();
-      // S = Phi22 - Phi21 K^T - K M over Phi22, upper triangle, mirrored
-      {
-        const int np = n2 * (n2 + 1) / 2;
-        int a = 0, b = lane;
-        while (a < n2 && b >= n2) { b += a + 1 - n2; ++a; }
-        for (int e = lane; e < np; e += 32) {
-          const double *fa = F + (m + a) * ldf, *ka = P + (m + a) * ldp, *kb = P + (m + b) * ldp;
-          double t = fa[m + b];
-          for (int l = 0; l < m; ++l) t = __fma_rn(-fa[l], kb[l], t);
-          for (int l = 0; l < m; ++l) t = __fma_rn(-ka[l], F[l * ldf + m + b], t);
-          F[(m + a) * ldf + m + b] = t;
-          F[(m + b) * ldf + m + a] = t;
-          b += 32;
-          while (a < n2 && b >= n2) { b += a + 1 - n2; ++a; }
-        }
-      }
-      __syncwarp();
-      // ---- S c2 = f2, LU with partial pivoting; f2 rides along.  Row k of S
-      // is row m + k of F; its reciprocal pivot goes to the diagonal.
-      double *S = F + m * ldf + m, *f2 = f + 3 * m;
-      for (int k = 0; k < n2; ++k) {
-        const int piv = pivot_row(S + k, ldf, k, n2, lane);
-        if (piv >= n2) { singular = true; break; }
-        if (piv != k) {
-          for (int c = k + lane; c < n2; c += 32) {
-            const double t = S[k * ldf + c];
-            S[k * ldf + c] = S[piv * ldf + c];
-            S[piv * ldf + c] = t;
-          }
-          if (lane < 3) {
-            const double t = f2[3 * k + lane];
-            f2[3 * k + lane] = f2[3 * piv + lane];
-            f2[3 * piv + lane] = t;
-          }
-          __syncwarp();
-        }
-        const double pk = S[k * ldf + k], kinv = __drcp_rn(pk);
-        for (int r = k + 1 + lane; r < n2; r += 32)
-          S[r * ldf + k] = ratio(S[r * ldf + k], pk, kinv);
-        __syncwarp();
-        if (lane == 0) S[k * ldf + k] = kinv;
-        rank_one(S, ldf, k, k + 1, n2, k + 1, n2, lane);
-        for (int e = lane; e < 3 * (n2 - 1 - k); e += 32) {
-          const int r = k + 1 + e / 3, s = e % 3;
-          f2[3 * r + s] = __fma_rn(-S[r * ldf + k], f2[3 * k + s], f2[3 * r + s]);
-        }
-        __syncwarp();
-      }
-      if (!singular) {
-        for (int j = n2 - 1; j >= 0; --j) {
-          if (lane < 3) f2[3 * j + lane] = __dmul_rn(f2[3 * j + lane], S[j * ldf + j]);
-          __syncwarp();
-          for (int e = lane; e < 3 * j; e += 32) {
-            const int r = e / 3, s = e % 3;
-            f2[e] = __fma_rn(-S[r * ldf + j], f2[3 * j + s], f2[e]);
-          }
-          __syncwarp();
-        }
-        // c1 = c_p - K^T c2
-        for (int e = lane; e < 3 * m; e += 32) {
-          const int l = e / 3, s = e % 3;
-          double t = g[e];
-          for (int b = 0; b < n2; ++b) t = __fma_rn(-P[(m + b) * ldp + l], f2[3 * b + s], t);
-          f[e] = t;
-        }
-        __syncwarp();
-      }
-    }
-    if (singular) {
-      for (int a = lane; a < q; a += 32) {
-        if (wx) wx[(int64_t)i * q + a] = 0.0;
-        if (wy) wy[(int64_t)i * q + a] = 0.0;
-        if (wl) wl[(int64_t)i * q + a] = 0.0;
-      }
-      if (lane == 0) atomicMin(first_singular, i);
-      __syncwarp();
-      continue;
-    }
-    const double h2inv = __drcp_rn(__dmul_rn(h, h));
-    for (int a = lane; a < q; a += 32) {
-      const int64_t o = (int64_t)i * q + ord[a];
-      if (wx) wx[o] = __dmul_rn(f[3 * a], hinv);
-      if (wy) wy[o] = __dmul_rn(f[3 * a + 1], hinv);
-      if (wl) wl[o] = __dmul_rn(f[3 * a + 2], h2inv);
+    rank_one<LW>(P, ldp, k, k + 1, q + 3, k + 1, m, lane);
+    __syncwarp();
+  }
+  // ---- K = L2 L1^-1 and c_p^T in place, a column at a time from the last
+  for (int j = m - 1; j > 0; --j) {
+    for (int e = lane; e < (n2 + 3) * j; e += LW) {
+      const int r = m + e / j, c = e - (e / j) * j;
+      P[r * ldp + c] = __fma_rn(-P[r * ldp + j], P[j * ldp + c], P[r * ldp + c]);
     }
     __syncwarp();
   }
+  // ---- Phi: r^3 of the permuted points, symmetric with a zero diagonal;
+  // the q(q-1)/2 pairs a < b dealt over the lanes in row-major order
+  for (int a = lane; a < q; a += LW) F[a * ldf + a] = 0.0;
+  {
+    // pair number e -> (a, b): past the end of row a (b >= q) it goes on
+    // at b - q positions into row a + 1, whose first pair is (a+1, a+2)
+    const int np = q * (q - 1) / 2;
+    int a = 0, b = 1 + lane;
+    while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
+    for (int e = lane; e < np; e += LW) {
+      const double dx = __dsub_rn(xi[a], xi[b]), dy = __dsub_rn(eta[a], eta[b]);
+      const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+      const double r3 = __dmul_rn(__dsqrt_rn(d2), d2);
+      F[a * ldf + b] = r3;
+      F[b * ldf + a] = r3;
+      b += LW;
+      while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
+    }
+  }
+  // right-hand sides: d/dxi, d/deta and Laplacian of r^3 about the centre
+  for (int a = lane; a < q; a += LW) {
+    const double xa = xi[a], ya = eta[a];
+    const double rj = __dsqrt_rn(__dadd_rn(__dmul_rn(xa, xa), __dmul_rn(ya, ya)));
+    const double r3 = __dmul_rn(3.0, rj);
+    double *f = F + a * ldf + q;
+    f[0] = __dmul_rn(r3, __dsub_rn(0.0, xa));
+    f[1] = __dmul_rn(r3, __dsub_rn(0.0, ya));
+    f[2] = __dmul_rn(9.0, rj);
+  }
+  __syncwarp();
+  // [M f1] = [Phi12 f1] - Phi11 [K^T c_p] over [Phi12 f1]
+  for (int e = lane; e < m * (n2 + 3); e += LW) {
+    const int a = e / (n2 + 3), b = e - a * (n2 + 3);
+    const double *kb = P + (m + b) * ldp, *fa = F + a * ldf;
+    double t = fa[m + b];
+    for (int l = 0; l < m; ++l) t = __fma_rn(-fa[l], kb[l], t);
+    F[a * ldf + m + b] = t;
+  }
+  __syncwarp();
+  // [S f2] = [Phi22 f2] - Phi21 [K^T c_p] - K [M f1] over [Phi22 f2], the
+  // upper triangle of S, mirrored
+  {
+    const int w = n2 + 3, np = n2 * (n2 + 1) / 2 + 3 * n2;
+    int a = 0, b = lane;
+    while (a < n2 && b >= w) { b += a + 1 - w; ++a; }
+    for (int e = lane; e < np; e += LW) {
+      const double *fa = F + (m + a) * ldf, *ka = P + (m + a) * ldp, *kb = P + (m + b) * ldp;
+      double t = fa[m + b];
+      for (int l = 0; l < m; ++l) t = __fma_rn(-fa[l], kb[l], t);
+      for (int l = 0; l < m; ++l) t = __fma_rn(-ka[l], F[l * ldf + m + b], t);
+      F[(m + a) * ldf + m + b] = t;
+      if (b < n2) F[(m + b) * ldf + m + a] = t;
+      b += LW;
+      while (a < n2 && b >= w) { b += a + 1 - w; ++a; }
+    }
+  }
+  __syncwarp();
+  // ---- S c2 = f2, LU with partial pivoting; f2 (three more columns) rides
+  // along.  Row k of S is row m + k of F; its reciprocal pivot goes to the
+  // diagonal.
+  double *S = F + m * ldf + m;
+  for (int k = 0; k < n2; ++k) {
+    int piv = pivot_row<LW>(S + k, ldf, k, n2, lane);
+    if (piv >= n2) { singular = true; piv = k; }
+    if (piv != k)
+      for (int c = k + lane; c < n2 + 3; c += LW) {
+        const double t = S[k * ldf + c];
+        S[k * ldf + c] = S[piv * ldf + c];
+        S[piv * ldf + c] = t;
+      }
+    __syncwarp();
+    const double pk = S[k * ldf + k], kinv = __drcp_rn(pk);
+    for (int r = k + 1 + lane; r < n2; r += LW)
+      S[r * ldf + k] = ratio(S[r * ldf + k], pk, kinv);
+    __syncwarp();
+    if (lane == 0) S[k * ldf + k] = kinv;
+    rank_one<LW>(S, ldf, k, k + 1, n2, k + 1, n2 + 3, lane);
+    __syncwarp();
+  }
+  for (int j = n2 - 1; j >= 0; --j) {
+    double *fj = S + j * ldf + n2;
+    if (lane < 3) fj[lane] = __dmul_rn(fj[lane], S[j * ldf + j]);
+    __syncwarp();
+    for (int e = lane; e < 3 * j; e += LW) {
+      const int r = e / 3, s = e % 3;
+      double *fr = S + r * ldf + n2 + s;
+      *fr = __fma_rn(-S[r * ldf + j], fj[s], *fr);
+    }
+    __syncwarp();
+  }
+  // c1 = c_p - K^T c2, over f1
+  for (int e = lane; e < 3 * m; e += LW) {
+    const int l = e / 3, s = e % 3;
+    double t = P[(q + s) * ldp + l];
+    for (int b = 0; b < n2; ++b) t = __fma_rn(-P[(m + b) * ldp + l], S[b * ldf + n2 + s], t);
+    F[l * ldf + q + s] = t;
+  }
+  __syncwarp();
+  if (out) {
+    const double h2inv = __drcp_rn(__dmul_rn(h, h));
+    for (int a = lane; a < q; a += LW) {
+      const int64_t o = (int64_t)i * q + ord[a];
+      const double *c = F + a * ldf + q;
+      if (wx) wx[o] = singular ? 0.0 : __dmul_rn(c[0], hinv);
+      if (wy) wy[o] = singular ? 0.0 : __dmul_rn(c[1], hinv);
+      if (wl) wl[o] = singular ? 0.0 : __dmul_rn(c[2], h2inv);
+    }
+    if (singular && lane == 0) atomicMin(first_singular, i);
+  }
 }
 
-int weights_config(int q, int degree, int *wpb, size_t *smem) {
+// Lanes a cloud of n (a block is one warp) and a block's shared memory.  The
+// fewest lanes that leave each SM more than nine warps by shared memory and
+// eight by n: with fewer the FP64 pipe waits for the steps' latencies.  Times
+// in us with 32, 16, 8 and 4 lanes: 40 000 clouds, q = 12, m = 6: 658, 425,
+// 347, 314 (11 warps with 4); q = 20, m = 10: 1188, 970, 922, 1386 (9.3 with
+// 8, 4.6 with 4); q = 28, m = 10: 2051, 1876, 2518 (11 with 16); q = 30,
+// m = 15: 2431, 2525 (9 with 16); q = 42, m = 21: 5691, 8368.  900 clouds,
+// q = 12: 54, 55, 64, 81; 3 600, q = 20, m = 10: 137, 125, 127, 178.
+// Blocks of 16 warps took 2 to 60% longer (2 500 clouds, q = 30: 327 us
+// against 200): a new block needs only one warp's clouds to end.
+int weights_config(int n, int q, int degree, int num_sms, int *lw, size_t *smem) {
   const int m = (degree + 1) * (degree + 2) / 2;
   const size_t per = (size_t)WeightsLayout(q, m).total * sizeof(double);
-  // as many warps as shared memory holds, up to 16 (q = 30: 16 x 13 KB):
-  // the FP64 pipe needs several warps per scheduler to hide the shared-
-  // memory latency in front of each update
-  int w = (int)((224 * 1024) / per);
-  if (w > 16) w = 16;
-  if (w < 1) return RBFFD_EINVAL;
-  *wpb = w;
-  *smem = per * w;
+  const int fit = (int)((224 * 1024) / per);  // clouds an SM
+  if (fit < 1) return RBFFD_EINVAL;
+  *lw = 4;
+  while (*lw < 32 && (fit * *lw <= 9 * 32 || (long long)n * *lw < 8LL * 32 * num_sms)) *lw *= 2;
+  *smem = per * (32 / *lw);
   return RBFFD_OK;
 }
 
 int weights_run(rbffd_ctx *ctx, int n, const double *x, const double *y, int q,
                 const int32_t *idx, int degree, double *wx, double *wy, double *wl,
                 int *d_first_singular, double Lx, double Ly) {
-  int m = (degree + 1) * (degree + 2) / 2;
-  RBFFD_TRY(ensure_tables(ctx->device));
-  int wpb;
+  const int m = (degree + 1) * (degree + 2) / 2;
+  int lw;
   size_t smem;
-  RBFFD_TRY(weights_config(q, degree, &wpb, &smem));
-  RBFFD_CK(cudaFuncSetAttribute(k_weights, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem));
-  int blocks = (n + wpb - 1) / wpb;
-  int cap = ctx->num_sms * 16;
-  if (blocks > cap) blocks = cap;
-  k_weights<<<blocks, 32 * wpb, smem, ctx->stream>>>(n, x, y, q, idx, m, wpb, wx, wy, wl,
+  RBFFD_TRY(weights_config(n, q, degree, ctx->num_sms, &lw, &smem));
+  const auto fn = lw == 4    ? k_weights<4>
+                  : lw == 8  ? k_weights<8>
+                  : lw == 16 ? k_weights<16>
+                             : k_weights<32>;
+  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int cpb = 32 / lw;
+  fn<<<(n + cpb - 1) / cpb, 32, smem, ctx->stream>>>(n, x, y, q, idx, m, degree, wx, wy, wl,
                                                      d_first_singular, Lx, Ly);
   return after_launch(ctx, "k_weights");
 }

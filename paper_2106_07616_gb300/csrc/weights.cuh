@@ -4,7 +4,7 @@
 
 namespace rbffd {
 int weights_check_args(int n, int q, int degree);
-int weights_config(int q, int degree, int *wpb, size_t *smem);
+int weights_config(int n, int q, int degree, int num_sms, int *lw, size_t *smem);
 // d_first_singular: device int, must hold INT_MAX on entry; receives the
 // lowest singular cloud index.
 // Lx, Ly: periods of the axes (0: bounded); cloud members enter at their
