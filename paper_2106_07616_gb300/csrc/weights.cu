@@ -111,7 +111,10 @@ __device__ __forceinline__ void rank_one(double *M, int ld, int k, int r0, int n
 // c_p^T by the steps that make K), f as three more columns of Phi.
 // At q = 2 m this takes 32 k flops for q = 30 instead of 73 k (two thirds of
 // (q + m)^3 and the right-hand sides).  A cloud is singular when either
-// factorisation meets an exactly zero pivot, as the augmented matrix is.
+// factorisation meets an exactly zero pivot, as the augmented matrix is; two
+// cases that there cancel exactly and here only up to rounding are looked for:
+// coinciding points (S is made by symmetry, which tells its two equal rows
+// apart) and points on one line through the centre (x and y are one column).
 // Lanes a cloud: a warp's clouds share the instructions that one lane would
 // do for all (reciprocals) and the part-filled last ones of every loop.
 template <int LW>
@@ -177,8 +180,19 @@ __global__ void __launch_bounds__(32)
     P[(q + s) * ldp + l] = s < 2 ? (l == s + 1 ? 1.0 : 0.0) : l == 3 || l == 5 ? 2.0 : 0.0;
   }
   __syncwarp();
+  // all on the line through the centre and the last point?
+  int off = degree < 1;
+  {
+    const double xl = xi[q - 1], yl = eta[q - 1];
+    for (int a = lane; a < q; a += LW)
+      off |= __double_as_longlong(__dsub_rn(__dmul_rn(xi[a], yl), __dmul_rn(xl, eta[a]))) << 1 != 0;
+    off |= ((__double_as_longlong(xl) | __double_as_longlong(yl)) << 1) == 0;
+  }
+#pragma unroll
+  for (int o = LW / 2; o > 0; o >>= 1) off |= __shfl_xor_sync(0xffffffffu, off, o);
+  __syncwarp();
   // ---- P = [L1; L2] U
-  bool singular = false;
+  bool singular = off == 0;
   for (int k = 0; k < m; ++k) {
     int piv = pivot_row<LW>(P + k, ldp, k, q, lane);
     if (piv >= q) { singular = true; piv = k; }
@@ -218,6 +232,7 @@ __global__ void __launch_bounds__(32)
   // ---- Phi: r^3 of the permuted points, symmetric with a zero diagonal;
   // the q(q-1)/2 pairs a < b dealt over the lanes in row-major order
   for (int a = lane; a < q; a += LW) F[a * ldf + a] = 0.0;
+  int twice = 0;  // two points in one place: two equal rows
   {
     // pair number e -> (a, b): past the end of row a (b >= q) it goes on
     // at b - q positions into row a + 1, whose first pair is (a+1, a+2)
@@ -226,6 +241,7 @@ __global__ void __launch_bounds__(32)
     while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
     for (int e = lane; e < np; e += LW) {
       const double dx = __dsub_rn(xi[a], xi[b]), dy = __dsub_rn(eta[a], eta[b]);
+      twice |= ((__double_as_longlong(dx) | __double_as_longlong(dy)) << 1) == 0;
       const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
       const double r3 = __dmul_rn(__dsqrt_rn(d2), d2);
       F[a * ldf + b] = r3;
@@ -234,6 +250,9 @@ __global__ void __launch_bounds__(32)
       while (a < q - 1 && b >= q) { b += a + 2 - q; ++a; }
     }
   }
+#pragma unroll
+  for (int o = LW / 2; o > 0; o >>= 1) twice |= __shfl_xor_sync(0xffffffffu, twice, o);
+  singular |= twice != 0;
   // right-hand sides: d/dxi, d/deta and Laplacian of r^3 about the centre
   for (int a = lane; a < q; a += LW) {
     const double xa = xi[a], ya = eta[a];

@@ -60,3 +60,17 @@ def test_singular_clouds_leave_their_neighbours(q, degree):
     for a, b in zip(got, regular):
         assert not a[broken].any()
         assert np.array_equal(a[rest], b[rest])
+
+
+@pytest.mark.parametrize("slope", [0.0, 1.0, -1.0, 2.0, -0.25])
+@pytest.mark.parametrize("q,degree", [(12, 2), (20, 3), (42, 5)])
+def test_points_of_a_line_are_singular(q, degree, slope):
+    """On y = slope x two columns of the polynomials are one, up to a power of
+    two: singular."""
+    r = np.random.Generator(np.random.PCG64(q))
+    x = np.sort(r.integers(-2**20, 2**20, 3000)).astype(np.float64)  # slope x exact
+    x = np.unique(x)
+    y = slope * x
+    bad, got = gpu_weights(x, y, oracle.knn(x, y, q), degree)
+    assert bad == 0
+    assert not any(a.any() for a in got)
