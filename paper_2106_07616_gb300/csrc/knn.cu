@@ -87,7 +87,8 @@ __device__ __forceinline__ Grid make_grid(const unsigned long long *bbox, int m)
   return g;
 }
 
-// one thread's grid for the block (FP64 divisions take over 400 cycles)
+// one thread's grid for the block (FP64 divisions take over 400 cycles); the
+// search, in blocks of four points, reads the one that k_cell_count leaves
 __device__ __forceinline__ const Grid &block_grid(const unsigned long long *bbox, int m) {
   __shared__ Grid g;
   if (threadIdx.x == 0) g = make_grid(bbox, m);
@@ -102,8 +103,9 @@ __device__ __forceinline__ int cell_coord(double v, double v0, double inv, int G
 
 __global__ void k_cell_count(int n, const double *__restrict__ x, const double *__restrict__ y,
                              const unsigned long long *bbox, int m, int *__restrict__ cell,
-                             int *__restrict__ cnt) {
+                             int *__restrict__ cnt, Grid *grid) {
   const Grid &g = block_grid(bbox, m);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *grid = g;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int c = cell_coord(y[i], g.y0, g.iy, g.Gy) * g.Gx + cell_coord(x[i], g.x0, g.ix, g.Gx);
@@ -166,19 +168,24 @@ __device__ __forceinline__ bool key_less(double da, int ja, double db, int jb) {
 // order (d^2, index), counted by every lane for its own: no sorting, no
 // local memory.  A thread with an insertion-sorted list per point was bound
 // by that list's local-memory traffic and by divergence: the whole search of
-// 147 827 graded points at q = 20 took 1.20 ms with it, 0.55 ms this way.
+// 147 827 graded points at q = 20 took 1.20 ms with it, 0.55 ms this way, and
+// 0.41 ms with the ranks counted by d^2 alone (the index decides only where a
+// place stays empty), two candidates a lane at once, and the grid's FP64
+// divisions made once instead of by every block of four points.  It is bound
+// by instruction issue and the FP64 distances (53% of the pipe before).
 // Points whose block holds more than CAP candidates at every usable r go to
 // the list `rest` (k_knn_query searches them).
 constexpr int KNN_CAP = 256;
 
 __global__ void __launch_bounds__(128) k_knn_warp(
     int n, const double *__restrict__ x, const double *__restrict__ y,
-    const int8_t *__restrict__ tag, int q, const unsigned long long *bbox, int m,
+    const int8_t *__restrict__ tag, int q, const Grid *__restrict__ grid,
     const int *__restrict__ start, const int *__restrict__ pts, int32_t *__restrict__ idx,
     int *err, int *nrest, int *__restrict__ rest, int r_first) {
-  __shared__ unsigned long long sd[4][KNN_CAP];
-  __shared__ int sj[4][KNN_CAP];
-  const Grid &g = block_grid(bbox, m);
+  __shared__ __align__(16) unsigned long long sd[4][KNN_CAP];
+  __shared__ int sj[4][KNN_CAP], sp[4][32], sa[4][32];
+  __shared__ uint16_t sr[4][KNN_CAP];
+  const Grid g = *grid;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * 4 + w, K = q - 1;
   if (i >= n) return;
@@ -210,22 +217,23 @@ __global__ void __launch_bounds__(128) k_knn_warp(
       if (lane >= d) pre += v;
     }
     const int M = __shfl_sync(0xffffffffu, pre, 31);
+    // run k ends before candidate sp[k]; candidate t of it is pts[sa[k] + t]
+    __syncwarp();
+    sp[w][lane] = lane < rows ? pre : 0x7fffffff;
+    sa[w][lane] = s - (pre - c);
+    __syncwarp();
+    int row = 0;
     const double clear = (double)r * cmin * (1.0 - 1e-9);
     const double lim = all ? __longlong_as_double(0x7ff0000000000000ll) : __dmul_rn(clear, clear);
     kept = 0;
     for (int t0 = 0; t0 < M; t0 += 32) {
       const int t = t0 + lane;
-      int at = 0;  // place in pts of candidate t
-      for (int k = 0; k < rows; ++k) {
-        const int pk = __shfl_sync(0xffffffffu, pre, k), ck = __shfl_sync(0xffffffffu, c, k),
-                  sk = __shfl_sync(0xffffffffu, s, k);
-        if (t < pk && t >= pk - ck) at = sk + t - (pk - ck);
-      }
       bool keep = false;
       double d2 = 0.0;
       int j = 0;
       if (t < M) {
-        j = __ldg(pts + at);
+        while (t >= sp[w][row]) ++row;
+        j = __ldg(pts + sa[w][row] + t);
         if (j != i && !(bnd && tag[j] != 0)) {
           const double dx = __dsub_rn(x[j], xi), dy = __dsub_rn(y[j], yi);
           d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
@@ -264,7 +272,40 @@ __global__ void __launch_bounds__(128) k_knn_warp(
     for (int s = lane; s < K; s += 32) idx[o + 1 + s] = i;
     return;
   }
-  // d^2 >= 0, so its bit pattern orders as its value
+  // d^2 >= 0, so its bit pattern orders as its value.  Ranks by d^2 alone, two
+  // candidates of a lane at once; where two are equal a place stays empty, and
+  // the ranks are counted again with the index
+  constexpr uint16_t EMPTY = 0xffff;
+  uint16_t *kr = sr[w];
+  for (int c = lane; c < kept; c += 32) kr[c] = EMPTY;
+  __syncwarp();
+  for (int c0 = 0; c0 < kept; c0 += 64) {
+    const int ca = c0 + lane, cb = ca + 32;
+    const unsigned long long da = ca < kept ? kd[ca] : 0ull, db = cb < kept ? kd[cb] : 0ull;
+    int ra = 0, rb = 0, k = 0;
+    for (; k + 2 <= kept; k += 2) {
+      const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(kd + k);
+      ra += d.x < da;
+      rb += d.x < db;
+      ra += d.y < da;
+      rb += d.y < db;
+    }
+    if (k < kept) {
+      ra += kd[k] < da;
+      rb += kd[k] < db;
+    }
+    if (ca < kept) kr[ra] = (uint16_t)ca;
+    if (cb < kept) kr[rb] = (uint16_t)cb;
+  }
+  __syncwarp();
+  bool tie = false;
+  for (int p = lane; p < kept; p += 32) {
+    const int c = kr[p];
+    tie |= c == EMPTY;
+    if (p < K && c != EMPTY) idx[o + 1 + p] = kj[c];
+  }
+  if (!__any_sync(0xffffffffu, tie)) return;
+  __syncwarp();
   for (int c = lane; c < kept; c += 32) {
     const unsigned long long dc = kd[c];
     const int jc = kj[c];
@@ -295,11 +336,11 @@ __device__ __forceinline__ int ring_index(int c, int d, int G, bool periodic) {
 template <int KMAX>
 __global__ void __launch_bounds__(128) k_knn_query(
     int n, const double *__restrict__ x, const double *__restrict__ y,
-    const int8_t *__restrict__ tag, int q, const unsigned long long *bbox, int m,
+    const int8_t *__restrict__ tag, int q, const Grid *__restrict__ grid,
     const int *__restrict__ start, const int *__restrict__ pts, int32_t *__restrict__ idx,
     int *err, const int *nrest, const int *rest, double Lx, double Ly) {
   if (rest != nullptr && blockIdx.x * blockDim.x >= *nrest) return;
-  const Grid &g = block_grid(bbox, m);
+  const Grid g = *grid;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (rest != nullptr ? *nrest : n)) return;
   if (rest != nullptr) i = rest[i];
@@ -379,6 +420,7 @@ int knn_workspace_bytes(int n, KnnLayout *lay) {
   lay->off_bbox = take(4 * sizeof(unsigned long long) + 2 * sizeof(int));
   lay->off_cnt = take((size_t)m * sizeof(int));
   lay->zero_bytes = off;
+  lay->off_grid = take(sizeof(Grid));
   lay->off_cell = take((size_t)n * sizeof(int));
   lay->off_start = take((size_t)(m + 1) * sizeof(int));
   lay->off_pts = take((size_t)n * sizeof(int));
@@ -391,6 +433,7 @@ int knn_run(rbffd_ctx *ctx, void *ws, const KnnLayout &lay, int n, const double 
   char *b = (char *)ws;
   unsigned long long *bbox = (unsigned long long *)(b + lay.off_bbox);
   int *err = (int *)(bbox + 4), *nrest = err + 1;
+  Grid *grid = (Grid *)(b + lay.off_grid);
   int *cell = (int *)(b + lay.off_cell);  // also, after the fill, the rest list
   int *cnt = (int *)(b + lay.off_cnt);
   int *start = (int *)(b + lay.off_start);
@@ -401,7 +444,7 @@ int knn_run(rbffd_ctx *ctx, void *ws, const KnnLayout &lay, int n, const double 
   const int nb = (n + 255) / 256;
   k_bbox<<<nb < 2 * ctx->num_sms ? nb : 2 * ctx->num_sms, 256, 0, st>>>(n, x, y, bbox);
   RBFFD_TRY(after_launch(ctx, "k_bbox"));
-  k_cell_count<<<nb, 256, 0, st>>>(n, x, y, bbox, m, cell, cnt);
+  k_cell_count<<<nb, 256, 0, st>>>(n, x, y, bbox, m, cell, cnt, grid);
   RBFFD_TRY(after_launch(ctx, "k_cell_count"));
   k_scan<<<(m + 1023) / 1024, 1024, 0, st>>>(cnt, start, m);
   RBFFD_TRY(after_launch(ctx, "k_scan"));
@@ -415,18 +458,18 @@ int knn_run(rbffd_ctx *ctx, void *ws, const KnnLayout &lay, int n, const double 
     int r_first = 1;
     while (6.2832 * r_first * r_first < q - 1) ++r_first;
     rest = cell;
-    k_knn_warp<<<(n + 3) / 4, 128, 0, st>>>(n, x, y, tag, q, bbox, m, start, pts, idx, err,
+    k_knn_warp<<<(n + 3) / 4, 128, 0, st>>>(n, x, y, tag, q, grid, start, pts, idx, err,
                                             nrest, rest, r_first);
     RBFFD_TRY(after_launch(ctx, "k_knn_warp"));
   }
   if (q - 1 <= 32) {
-    k_knn_query<32><<<qb, 128, 0, st>>>(n, x, y, tag, q, bbox, m, start, pts, idx, err, nrest,
+    k_knn_query<32><<<qb, 128, 0, st>>>(n, x, y, tag, q, grid, start, pts, idx, err, nrest,
                                         rest, Lx, Ly);
   } else if (q - 1 <= 64) {
-    k_knn_query<64><<<qb, 128, 0, st>>>(n, x, y, tag, q, bbox, m, start, pts, idx, err, nrest,
+    k_knn_query<64><<<qb, 128, 0, st>>>(n, x, y, tag, q, grid, start, pts, idx, err, nrest,
                                         rest, Lx, Ly);
   } else {
-    k_knn_query<128><<<qb, 128, 0, st>>>(n, x, y, tag, q, bbox, m, start, pts, idx, err, nrest,
+    k_knn_query<128><<<qb, 128, 0, st>>>(n, x, y, tag, q, grid, start, pts, idx, err, nrest,
                                          rest, Lx, Ly);
   }
   RBFFD_TRY(after_launch(ctx, "k_knn_query"));
