@@ -119,6 +119,7 @@ void dev_release(rbffd_ctx *ctx, size_t bytes);
 // Kept between calls -- cudaMalloc and cudaFree cost 0.1 ms and more a call --
 // up to 64 MB; a larger one replaces it and is given back at the next call.
 int ctx_scratch(rbffd_ctx *ctx, size_t bytes, void **out);
+void ctx_scratch_free(rbffd_ctx *ctx);
 // Small pinned host buffer of at least `bytes` (owned by the context).
 int pinned(rbffd_ctx *ctx, size_t bytes, void **out);
 

@@ -51,14 +51,19 @@ void dev_free(rbffd_ctx *ctx, void *p, size_t bytes) {
   dev_release(ctx, bytes);
 }
 
+void ctx_scratch_free(rbffd_ctx *ctx) {
+  if (!ctx->scratch) return;
+  cudaStreamSynchronize(ctx->stream);
+  dev_free(ctx, ctx->scratch, ctx->scratch_bytes);
+  ctx->scratch = nullptr;
+  ctx->scratch_bytes = 0;
+}
+
 int ctx_scratch(rbffd_ctx *ctx, size_t bytes, void **out) {
   *out = nullptr;
   constexpr size_t KEEP = (size_t)64 << 20;
   if (ctx->scratch_bytes < bytes || (ctx->scratch_bytes > KEEP && bytes <= KEEP)) {
-    cudaStreamSynchronize(ctx->stream);
-    dev_free(ctx, ctx->scratch, ctx->scratch_bytes);
-    ctx->scratch = nullptr;
-    ctx->scratch_bytes = 0;
+    ctx_scratch_free(ctx);
     RBFFD_TRY(dev_alloc(ctx, &ctx->scratch, bytes));
     ctx->scratch_bytes = bytes;
   }

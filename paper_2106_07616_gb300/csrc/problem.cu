@@ -719,6 +719,7 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       o_part32 = c.take<char>(krylov_ir_partials_inner_bytes(2, kb, P->inner));
     }
     size_t o_hl = 0, o_hi = 0, o_li = 0, o_rp = 0;
+    const size_t streaming = c.off;
     if (P->res.nb > 0) {
       o_hl = c.take<int32_t>((size_t)P->res.nb * P->res.hstride);
       o_hi = c.take<int32_t>(2 * (size_t)P->res.nb);
@@ -727,6 +728,16 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
     }
     P->bytes = c.off;
     int rc = dev_alloc(ctx, &P->mem, P->bytes);
+    if (rc == RBFFD_ENOMEM) {
+      // the context's own workspace goes first, then the resident solves
+      ctx_scratch_free(ctx);
+      rc = dev_alloc(ctx, &P->mem, P->bytes);
+    }
+    if (rc == RBFFD_ENOMEM && P->res.nb > 0) {
+      P->res = ResPlan();
+      P->bytes = streaming;
+      rc = dev_alloc(ctx, &P->mem, P->bytes);
+    }
     if (rc != RBFFD_OK) {
       delete P;
       ctx_unref(ctx);

@@ -109,3 +109,26 @@ def test_resident_batch_matches_oracle(name, precond):
     B.close()
     for P in probs:
         P.close()
+
+
+def test_tight_budget_runs_the_streaming_solves():
+    """A budget that holds a problem but not the resident solves' lists, with a
+    workspace kept by the context: the problem is made without them."""
+    import torch
+
+    fp = CASES["cluster_full"]()
+    full = rbffd.Problem(ctx(), fp)
+    budget = full.nbytes - 1
+    C = rbffd.Context(0, hbm_budget=budget)
+    full.close()
+    d = [torch.as_tensor(a, device="cuda:0") for a in (fp.x, fp.y, fp.tag)]
+    idx = torch.zeros((fp.n, fp.q), dtype=torch.int32, device="cuda:0")
+    rbffd.rbffd_build_stencils(C, *d, fp.q, idx)
+    P = rbffd.Problem(C, fp)
+    assert P.nbytes <= budget
+    O = oracle.Problem(fp, krylov_tol=1e-12, krylov_maxit=100000)
+    P.simple_iterate(fp.dt, krylov_tol=1e-12, krylov_maxit=100000)
+    O.simple_iterate(fp.dt)
+    for k in FIELDS:
+        assert rel_l2(P.get(k), O.get(k)) <= 1e-8, k
+    P.close()
