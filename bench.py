@@ -684,7 +684,7 @@ def run_native(args):
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": krylov_traffic(args.precision, args.workload, args.precond),
             "peak_source": peak_src,
-            "kernel": ("k_fgmres<1024> (pressure-correction flexible GMRES(30), FP32 multigrid "
+            "kernel": ("k_fgmres_res (pressure-correction flexible GMRES(30), FP32 multigrid "
                        "V-cycle preconditioner, persistent)" if args.precond == "fgmres" else
                        "k_bicgstab_amg<1024> (pressure-correction BiCGSTAB, multigrid "
                        "V-cycle preconditioner, persistent)" if args.precond == "amg" and

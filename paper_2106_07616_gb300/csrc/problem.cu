@@ -226,6 +226,7 @@ int build(rbffd_problem *P, const rbffd_problem_desc *d) {
   memset(P->res_hm, 0, sizeof(P->res_hm));
   if (ctx->prof) {
     const double N = P->q + (P->degree + 1) * (P->degree + 2) / 2;
+    // of the augmented elimination; the kernel's null space takes fewer
     const double flops = 2.0 * N * N * N / 3.0 + 6.0 * N * N + 10.0 * P->q * P->q;
     prof_collect(ctx, 3, RBFFD_KSTAT_KNN, P->n, 24.0 * P->n);
     prof_collect(ctx, 0, RBFFD_KSTAT_WEIGHTS, P->n, flops * P->n);

@@ -22,9 +22,13 @@
 // by rounding only, well inside the 1e-10 they are held to.  Measured on
 // GB300: 40 000 clouds at q = 30, degree 4 in 5.8 ms by elimination of the
 // augmented matrix, 3.2 ms by the null space with a warp a cloud and 16 warps a
-// block, 2.4 ms now: some 1 200 FP64 instructions a cloud, 19 000 cycles, keep
-// the pipe busy (error against 64-bit LAPACK 8e-14 and 1.3e-13 relative);
-// 10 201 clouds at q = 12, degree 2 in 0.47, 0.25 and 0.11 ms.
+// block, 2.5 ms now: some 1 200 FP64 instructions a cloud, 19 000 cycles, keep
+// the pipe busy (89% of its cycles); 10 201 clouds at q = 12, degree 2 in 0.47,
+// 0.25 and 0.11 ms.  Relative error against 80-bit elimination, augmented and
+// null space, worst of the three operators: degree 2 8.9e-15 and 7.8e-15,
+// degree 3 3.9e-14 and 4.4e-14, degree 4 1.1e-13 and 1.3e-13 (graded cylinder
+// 6.5e-14 and 9.3e-14), degree 5 4.1e-13 and 4.0e-13; 64-bit elimination with
+// another order of its sums lies as far apart (1.4e-13 at degree 4).
 #include "abi_guard.cuh"
 #include "common.cuh"
 #include "weights.cuh"
