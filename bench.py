@@ -100,8 +100,8 @@ KRYLOV_PROFILES = {
     "amg": ("k_bicgstab_amg_fp64_cavity200.md",
             ("krylov.cu", "krylov_dev.cuh", "common.cuh", "amg_dev.cuh", "amg.cuh", "amg.cu",
              "amg_setup.cu")),
-    "fgmres": ("k_fgmres_cavity200.md",
-               ("fgmres.cu", "fgmres.cuh", "krylov_dev.cuh", "common.cuh", "amg_dev.cuh",
+    "fgmres": ("k_fgmres_res_cavity200.md",
+               ("fgmres_res.cu", "fgmres.cuh", "resident.cu", "resident.cuh", "common.cuh",
                 "amg.cuh", "amg.cu", "amg_setup.cu")),
 }
 
