@@ -611,9 +611,9 @@ static int launch_resident(BatchScratch &S, int slot, int nr, const std::vector<
     a.flags = dflags + i;  // one arrival counter per system
     a.bar = dbars + i;
     // a member's second single system (symmetry lines) sums in the second
-    // half of the member's partials
+    // share of the member's partials
     const bool second = i > 0 && probs[i - 1] == probs[i];
-    a.res.part = (char *)probs[i]->res.part + (second ? RES_PART_BYTES / 2 : 0);
+    a.res.part = (char *)probs[i]->res.part + (second ? RES_SHARE_BYTES : 0);
     member_args(i, a, hb + S.off_sys[slot] + bytes * i, &need);
     smem = std::max(smem, need);
   }

@@ -65,17 +65,20 @@ struct FgState {
 // Products of one step summed over the team: warp d < D holds its CTA's
 // part; totals to tot[0..D).
 __device__ __forceinline__ bool products(res::Team &t, float s, int D, float *tot, float *cpart,
-                                         float *gpart) {
+                                         void *gpart) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int half = (t.epoch & 1) ? 32 : 0;
+  const unsigned int ep = t.epoch;  // of this exchange, before its barrier
+  auto at = [&](int v, int b) {
+    return reinterpret_cast<float *>(static_cast<char *>(gpart) + res_slot(ep, v, b, 4));
+  };
   if (w < D) {
     if (t.nb == 1) {
       if (lane == 0) tot[w] = s;
     } else if (t.cluster) {
-      float *slot = cpart + (half + w) * RES_CLUSTER + t.lb;
-      if (lane < t.nb) *res::cg::this_cluster().map_shared_rank(slot, lane) = s;
+      float *dst = cpart + res_cluster_slot(ep, 32, w, t.lb);
+      if (lane < t.nb) *res::cg::this_cluster().map_shared_rank(dst, lane) = s;
     } else if (lane == 0) {
-      gpart[(half + w) * RES_MAXB + t.lb] = s;
+      *at(w, t.lb) = s;
     }
   }
   const bool ok = res::team_barrier(t);
@@ -83,13 +86,12 @@ __device__ __forceinline__ bool products(res::Team &t, float s, int D, float *to
     if (w < D) {
       float r = 0.0f;
       if (t.cluster) {
-        if (lane < t.nb) r = cpart[(half + w) * RES_CLUSTER + lane];
+        if (lane < t.nb) r = cpart[res_cluster_slot(ep, 32, w, lane)];
       } else {
         float p[RES_MAXB / 32];
 #pragma unroll
         for (int u = 0; u < RES_MAXB / 32; ++u)
-          p[u] = lane + 32 * u < t.nb ? __ldcg(gpart + (half + w) * RES_MAXB + lane + 32 * u)
-                                      : 0.0f;
+          p[u] = lane + 32 * u < t.nb ? __ldcg(at(w, lane + 32 * u)) : 0.0f;
 #pragma unroll
         for (int u = 0; u < RES_MAXB / 32; ++u) r += p[u];
       }
@@ -128,8 +130,6 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
   float *Bs = reinterpret_cast<float *>(dyn + A.o_b);
   int2 *Rs = reinterpret_cast<int2 *>(dyn + A.o_r), *Ps = reinterpret_cast<int2 *>(dyn + A.o_p);
   float *ws = Vs + (size_t)A.kv * A.ldv;                    // w on the own rows (one more stride)
-  double *p64 = reinterpret_cast<double *>(A.res.part);
-  float *pf = reinterpret_cast<float *>(p64 + 2 * 2 * RES_MAXB);
   const int kv = A.kv, ldv = A.ldv;
 
   for (int e = tid; e < L; e += RES_NT) {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
       acc[0] = bi * bi;
       acc[1] = ri * ri;
     }
-    if (!res::team_totals<2>(team, acc, tot64, wsum64, cpart64, p64)) return false;
+    if (!res::team_totals<2, 2>(team, acc, tot64, wsum64, cpart64, A.res.part)) return false;
     if (tid == 0) {
       if (first) st.bnorm = sqrt(tot64[0]);
       st.beta = sqrt(tot64[1]);
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
         if (row.lead) ws[row.rl] = s;
       }
       __syncthreads();
-      if (!products(team, dots(j), j + 2, tot, cpart, pf)) { ok = false; break; }
+      if (!products(team, dots(j), j + 2, tot, cpart, A.res.part)) { ok = false; break; }
       {
         const float s = combine(j);
         if (tid <= j) H[tid + LDH * j] = tot[tid];
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_fgmres_res(const __grid_constant_
       }
       __syncthreads();
       // ---- second pass; u is published by its exchange
-      if (!products(team, dots(j), j + 2, tot, cpart, pf)) { ok = false; break; }
+      if (!products(team, dots(j), j + 2, tot, cpart, A.res.part)) { ok = false; break; }
       // h_{j+1,j} = sqrt((u, u) - sum c_i^2), by every warp in the same order
       float hn;
       {

@@ -769,8 +769,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
         }
         pubt[row.i] = rf;
       }
-      ok = res::team_totals<3 * NR>(team, acc, tot64, wsum64, cpart64,
-                                     reinterpret_cast<double *>(A.res.part));
+      ok = res::team_totals<3 * NR, 3 * NR>(team, acc, tot64, wsum64, cpart64, A.res.part);
       if (!ok) break;
       if (tid == 0) {
         int any = 0;
@@ -912,8 +911,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           }
           pubv[row.i] = vn;
         }
-        ok = res::team_totals<2 * NR>(team, acc, tot, wsum, cpart,
-                                      reinterpret_cast<PT *>(A.res.part));
+        ok = res::team_totals<2 * NR, 5 * NR>(team, acc, tot, wsum, cpart, A.res.part);
       }
       if (!ok) break;
       if (tid < NR && co.run[tid]) {
@@ -985,8 +983,7 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
           }
           pubt[row.i] = tn;
         }
-        ok = res::team_totals<5 * NR>(team, acc, tot, wsum, cpart,
-                                      reinterpret_cast<PT *>(A.res.part));
+        ok = res::team_totals<5 * NR, 5 * NR>(team, acc, tot, wsum, cpart, A.res.part);
       }
       if (!ok) break;
       if (tid < 32) {

@@ -90,7 +90,6 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
   const int R = K.res.R, r0 = min(n, lb * R), r1 = min(n, r0 + R), nr = r1 - r0;
   const int hm = K.res.hmax;
   res::Team team{K.flags, &K.bar->err, lb, nb, K.res.cluster, 0u};
-  double *part = reinterpret_cast<double *>(K.res.part);
   double *val = reinterpret_cast<double *>(dyn + A.o_val);
   uint16_t *idx = reinterpret_cast<uint16_t *>(dyn + A.o_idx);
   int *list = reinterpret_cast<int *>(dyn + A.o_list);
@@ -395,7 +394,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
             acc[2 * k + 1] = ri * ri;
           }
       }
-      ok = res::team_totals<2 * NR>(team, acc, tot, wsum, cpart, part, active);
+      ok = res::team_totals<2 * NR, VC>(team, acc, tot, wsum, cpart, K.res.part, active);
       if (!ok) break;
       if (tid < NR && ks[tid].state == KRY_RUNNING && ks[tid].need_init) {
         Scalars &c = ks[tid];
@@ -529,7 +528,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
           acc[3 * k + 2] = rh * r;
         }
       }
-      ok = res::team_totals<VA>(team, acc, tot, wsum, cpart, part, active);
+      ok = res::team_totals<VA, VC>(team, acc, tot, wsum, cpart, K.res.part, active);
     }
     if (!ok) break;
     if (tid < NR && ks[tid].run) {
@@ -638,7 +637,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
           acc[5 * k + 4] = rh * at[k];
         }
       }
-      ok = res::team_totals<VC>(team, acc, tot, wsum, cpart, part, active);
+      ok = res::team_totals<VC, VC>(team, acc, tot, wsum, cpart, K.res.part, active);
     }
     if (!ok) break;
     if (tid < 32) {

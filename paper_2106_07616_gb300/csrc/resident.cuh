@@ -44,8 +44,23 @@ struct ResPlan {
   const uint16_t *lidx = nullptr;   // ELL [q][ldn]: an entry's place in its CTA's list
   void *part = nullptr;             // RES_PART_BYTES of partial sums
 };
-// partial sums of a grid team: two halves of up to 64 values of 8 bytes
-constexpr size_t RES_PART_BYTES = 2 * 64 * RES_MAXB * 8;
+// Partial sums of a grid team: two shares (a pair of single systems on one
+// problem's memory takes one each) of two halves of up to 32 values of 8
+// bytes.  Alternate exchanges of a solve use alternate halves, at offsets
+// that no exchange's number of values or their type moves.
+constexpr size_t RES_HALF_BYTES = 32 * RES_MAXB * 8;
+constexpr size_t RES_SHARE_BYTES = 2 * RES_HALF_BYTES;
+constexpr size_t RES_PART_BYTES = 2 * RES_SHARE_BYTES;
+// Byte offset of value v of CTA b in the partial sums of exchange `epoch`
+// whose values have `bytes` each.
+__host__ __device__ constexpr size_t res_slot(unsigned int epoch, int v, int b, size_t bytes) {
+  return (epoch & 1) * RES_HALF_BYTES + ((size_t)v * RES_MAXB + b) * bytes;
+}
+// The same for a cluster team's array in shared memory, halves of vmax values
+// (the most of any exchange on that array), counted in values.
+__host__ __device__ constexpr int res_cluster_slot(unsigned int epoch, int vmax, int v, int b) {
+  return ((int)(epoch & 1) * vmax + v) * RES_CLUSTER + b;
+}
 
 // Team sizes a batched resident launch chooses from, and for a problem the
 // longest halo list at each (0: the team would not fit its rows).
@@ -184,31 +199,39 @@ __device__ __forceinline__ bool team_barrier(Team &t) {
 // Totals over the team of V values per thread, into tot[0..V) (shared; all
 // threads may read it on return), with a team barrier on the way.  Sums run
 // in a fixed order: every CTA gets bit-identical totals.  wsum: V x 32
-// shared; cpart: 2 x V x RES_CLUSTER shared (cluster teams); gpart: 2 x V x
-// RES_MAXB global (grid teams).  The two halves of the partial arrays serve
-// alternate exchanges, so a CTA may write the next partials while another
-// still reads these.
-template <int V, typename P>
+// shared; cpart: 2 x VMAX x RES_CLUSTER shared (cluster teams), VMAX the most
+// values of any exchange on that array; gpart: RES_SHARE_BYTES global (grid
+// teams), for exchanges of any type and number of values.  A CTA that has
+// left exchange e writes the partials of e + 1 while a slower one still reads
+// those of e; it reaches e + 2 only after every CTA has arrived at e + 1, so
+// after all reads of e.  Two halves are enough, then, as long as they are
+// disjoint for every V and type of the exchanges that share the array.
+template <int V, int VMAX, typename P>
 __device__ __forceinline__ bool team_totals(Team &t, P (&val)[pow2_ge(V)], P *tot, P *wsum,
-                                            P *cpart, P *gpart, bool active = true) {
+                                            P *cpart, void *gpart, bool active = true) {
   constexpr int VP = pow2_ge(V);
+  static_assert(V <= VMAX, "a half of the cluster's array holds VMAX values");
+  static_assert(res_slot(0, V, 0, sizeof(P)) <= RES_HALF_BYTES, "a half holds the values");
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (active) warp_totals<V>(val);
   else val[0] = P(0);
   if ((lane & (32 / VP - 1)) == 0 && lane / (32 / VP) < V)
     wsum[(lane / (32 / VP)) * 32 + w] = val[0];
   __syncthreads();
-  const int half = (t.epoch & 1) ? V : 0;
+  const unsigned int ep = t.epoch;  // of this exchange, before its barrier
+  auto slot = [&](int v, int b) {
+    return reinterpret_cast<P *>(static_cast<char *>(gpart) + res_slot(ep, v, b, sizeof(P)));
+  };
   if (w < V) {
     P s = lane < nw ? wsum[w * 32 + lane] : P(0);
     s = warp_total(s);
     if (t.nb == 1) {
       if (lane == 0) tot[w] = s;
     } else if (t.cluster) {
-      P *slot = cpart + (half + w) * RES_CLUSTER + t.lb;
-      if (lane < t.nb) *cg::this_cluster().map_shared_rank(slot, lane) = s;
+      P *dst = cpart + res_cluster_slot(ep, VMAX, w, t.lb);
+      if (lane < t.nb) *cg::this_cluster().map_shared_rank(dst, lane) = s;
     } else if (lane == 0) {
-      gpart[(half + w) * RES_MAXB + t.lb] = s;
+      *slot(w, t.lb) = s;
     }
   }
   const bool ok = team_barrier(t);
@@ -216,12 +239,12 @@ __device__ __forceinline__ bool team_totals(Team &t, P (&val)[pow2_ge(V)], P *to
     if (w < V) {
       P s = P(0);
       if (t.cluster) {
-        if (lane < t.nb) s = cpart[(half + w) * RES_CLUSTER + lane];
+        if (lane < t.nb) s = cpart[res_cluster_slot(ep, VMAX, w, lane)];
       } else {
         P p[RES_MAXB / 32];
 #pragma unroll
         for (int u = 0; u < RES_MAXB / 32; ++u)
-          p[u] = lane + 32 * u < t.nb ? ld_l2(gpart + (half + w) * RES_MAXB + lane + 32 * u) : P(0);
+          p[u] = lane + 32 * u < t.nb ? ld_l2(slot(w, lane + 32 * u)) : P(0);
 #pragma unroll
         for (int u = 0; u < RES_MAXB / 32; ++u) s += p[u];
       }
