@@ -1040,6 +1040,9 @@ __global__ void __launch_bounds__(RES_NT, 1) k_ir_res(const MixedArgs A) {
             if (fin[k])
               d[e].x[k] = IA::axpy(d[e].x[k], co.alp[k], IA::mul(p[own + e].x[k], di));
         }
+        // where the other system goes on, its phase A rewrites whole entries
+        // of d and p from other threads
+        __syncthreads();
       }
     }
     if (!ok) break;
