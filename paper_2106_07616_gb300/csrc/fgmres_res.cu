@@ -584,7 +584,7 @@ bool fg_layout(FgResArgs &a, size_t *smem) {
     at += round16(bytes);
     return (int)o;
   };
-  const size_t limit = 200 * 1024;
+  const size_t limit = RES_SMEM;
   a.o_list = take(4 * (size_t)hm);
   a.o_w = take(4 * (size_t)hm);
   a.o_work = take(8 * (size_t)hm);

@@ -1098,7 +1098,7 @@ const void *ir_res_kernel(int nr, int inner, bool ff_sums, int q, const ResPlan 
   const size_t s = inner == INNER_FF ? 8 : 4;
   if (s * nr * p.hmax > 65535) return nullptr;
   *smem = ir_res_halo_bytes(s, nr, p) + 8 * (size_t)nr * p.R;
-  if (*smem > 200 * 1024) return nullptr;
+  if (*smem > RES_SMEM) return nullptr;
   if (inner == INNER_FF)
     return nr == 1 ? ir_res_fn<1, ArithFF, ff>(E) : ir_res_fn<2, ArithFF, ff>(E);
   if (nr == 2) return ir_res_fn<2, ArithF32, float>(E);

@@ -726,7 +726,6 @@ __global__ void __launch_bounds__(RES_NT, 1)
 }
 
 int round16(size_t v) { return (int)((v + 15) / 16 * 16); }
-constexpr size_t SMEM_LIMIT = 200 * 1024;
 
 // Lanes a row: enough threads to hide the products' latency, no more (a
 // row sum's FP64 instructions grow with them).
@@ -755,14 +754,14 @@ bool layout(BicgResArgs &a, int nr, bool amg, size_t *smem) {
   // the list's scratch lies over what is loaded after it
   a.o_tmp = (int)at;
   const size_t tmp = p.hlist ? 0 : 8 * (size_t)((a.k.n + 31) / 32);
-  if (at + tmp > SMEM_LIMIT) return false;
-  a.vres = at + 8 * (size_t)q * a.ld <= SMEM_LIMIT;
+  if (at + tmp > RES_SMEM) return false;
+  a.vres = at + 8 * (size_t)q * a.ld <= RES_SMEM;
   if (a.vres) a.o_val = take(8 * (size_t)q * a.ld);
   if (amg) {
     const size_t bb = a.B ? 8 * (size_t)R1 * a.ldb : 0;
-    a.bres = a.B && at + bb <= SMEM_LIMIT;
+    a.bres = a.B && at + bb <= RES_SMEM;
     if (a.bres) a.o_b = take(bb);
-    const size_t left = at < SMEM_LIMIT ? SMEM_LIMIT - at : 0;
+    const size_t left = at < RES_SMEM ? RES_SMEM - at : 0;
     a.rcap = a.pcap = (int)(left / 2 / 12) / 4 * 4;
     a.o_rv = take(8 * (size_t)a.rcap);
     a.o_rc = take(4 * (size_t)a.rcap);
@@ -876,7 +875,7 @@ int krylov_res_batch_launch(rbffd_ctx *ctx, int nr, bool amg, int nctas, const v
   const void *fn = amg       ? (const void *)k_bicg_res_batch<1, true>
                    : nr == 1 ? (const void *)k_bicg_res_batch<1, false>
                              : (const void *)k_bicg_res_batch<2, false>;
-  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
   void *kargs[] = {(void *)&d_sys, (void *)&d_cta_team, (void *)&d_info};
   const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nctas), dim3(RES_NT), kargs, smem,
                                                     ctx->stream);

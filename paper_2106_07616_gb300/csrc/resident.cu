@@ -145,7 +145,7 @@ int res_halo_build(rbffd_ctx *ctx, const ResPlan &p, int n, int q, int ldn, cons
 
 int res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, size_t smem,
                const char *what) {
-  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nb);
   cfg.blockDim = dim3(RES_NT);

@@ -31,6 +31,11 @@ constexpr int RES_CLUSTER = 16;     // most CTAs of a cluster team
 constexpr int RES_CLUSTER_N = 4096; // most rows of a cluster team
 constexpr int RES_HCAP = 8192;      // largest halo list (16-bit byte offsets of 8-byte entries)
 constexpr int RES_MAXN = 150 * RES_NT;  // rows a team can own, one lane each
+// Most dynamic shared memory of a resident launch.  Every launch allows its
+// kernel this much, whatever it uses itself: the allowance belongs to the
+// function on the device, and another context's thread that lowered it
+// between this one's call and its launch would have the launch refused.
+constexpr int RES_SMEM = 200 * 1024;
 
 // The team's rows and halo lists of one problem (device arrays; plan on the host).
 struct ResPlan {

@@ -349,6 +349,10 @@ __global__ void __launch_bounds__(32)
   }
 }
 
+// Shared memory an SM's clouds may take, and what every launch allows its
+// kernel (resident.cuh: RES_SMEM says why not its own need).
+constexpr int WEIGHTS_SMEM = 224 * 1024;
+
 // Lanes a cloud of n (a block is one warp) and a block's shared memory.  The
 // fewest lanes that leave each SM more than nine warps by shared memory and
 // eight by n: with fewer the FP64 pipe waits for the steps' latencies.  Times
@@ -362,7 +366,7 @@ __global__ void __launch_bounds__(32)
 int weights_config(int n, int q, int degree, int num_sms, int *lw, size_t *smem) {
   const int m = (degree + 1) * (degree + 2) / 2;
   const size_t per = (size_t)WeightsLayout(q, m).total * sizeof(double);
-  const int fit = (int)((224 * 1024) / per);  // clouds an SM
+  const int fit = (int)(WEIGHTS_SMEM / per);  // clouds an SM
   if (fit < 1) return RBFFD_EINVAL;
   *lw = 4;
   while (*lw < 32 && (fit * *lw <= 9 * 32 || (long long)n * *lw < 8LL * 32 * num_sms)) *lw *= 2;
@@ -381,7 +385,7 @@ int weights_run(rbffd_ctx *ctx, int n, const double *x, const double *y, int q,
                   : lw == 8  ? k_weights<8>
                   : lw == 16 ? k_weights<16>
                              : k_weights<32>;
-  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, WEIGHTS_SMEM));
   const int cpb = 32 / lw;
   fn<<<(n + cpb - 1) / cpb, 32, smem, ctx->stream>>>(n, x, y, q, idx, m, degree, wx, wy, wl,
                                                      d_first_singular, Lx, Ly);
