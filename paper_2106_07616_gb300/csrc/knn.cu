@@ -56,7 +56,11 @@ __global__ void __launch_bounds__(256) k_bbox(int n, const double *__restrict__ 
 // cylinder cloud's 2:1 box, cells of the box's own shape doubled the
 // candidates).
 struct Grid {
-  double x0, y0, cx, cy, ix, iy;  // origin, cell sides and their reciprocals
+  double x0, y0, ix, iy;  // origin, reciprocals of the cell sides
+  // squares of the cells' sides, and of the smaller one, less what rounding may
+  // move a point against the cells' edges: no point r cells away or more has a
+  // smaller squared distance than r^2 times this
+  double cx2, cy2, c2;
   int Gx, Gy;
 };
 
@@ -78,13 +82,27 @@ __device__ __forceinline__ Grid make_grid(const unsigned long long *bbox, int m)
   if (!(gx >= 1.0)) gx = 1.0;
   g.Gx = gx < (double)m ? (int)gx : m;
   g.Gy = max(1, m / g.Gx);
-  g.cx = w / g.Gx;
-  g.cy = h / g.Gy;
-  if (!(g.cx > 0.0)) g.cx = 1.0;
-  if (!(g.cy > 0.0)) g.cy = 1.0;
-  g.ix = 1.0 / g.cx;
-  g.iy = 1.0 / g.cy;
+  double cx = w / g.Gx, cy = h / g.Gy;
+  if (!(cx > 0.0)) cx = 1.0;
+  if (!(cy > 0.0)) cy = 1.0;
+  g.ix = 1.0 / cx;
+  g.iy = 1.0 / cy;
+  cx *= 1.0 - (1e-9 + 1e-15 * g.Gx);
+  cy *= 1.0 - (1e-9 + 1e-15 * g.Gy);
+  g.cx2 = cx * cx;
+  g.cy2 = cy * cy;
+  g.c2 = fmin(g.cx2, g.cy2);
   return g;
+}
+
+// Points outside the searched block, r cells around the point's own, have at
+// least this squared distance: an axis along which the block holds every cell
+// does not count.  (With the smaller of the two sides for both axes, a search in a
+// box far longer than the grid could follow -- points on a line up to rounding
+// -- walked every ring of the long axis.)
+__device__ __forceinline__ double clearance2(const Grid &g, int r, bool all_x, bool all_y) {
+  if (all_x && all_y) return __longlong_as_double(0x7ff0000000000000ll);
+  return (double)r * (double)r * (all_x ? g.cy2 : all_y ? g.cx2 : g.c2);
 }
 
 // one thread's grid for the block (FP64 divisions take over 400 cycles); the
@@ -195,15 +213,16 @@ __global__ void __launch_bounds__(128) k_knn_warp(
   const double xi = x[i], yi = y[i];
   const bool bnd = tag != nullptr && tag[i] != 0;
   const int ci = cell_coord(xi, g.x0, g.ix, g.Gx), cj = cell_coord(yi, g.y0, g.iy, g.Gy);
-  const double cmin = fmin(g.cx, g.cy);
   unsigned long long *kd = sd[w];
   int *kj = sj[w];
-  int kept = 0, lo = 0;  // lo: the largest r known to hold too few
+  int kept = 0;
+  int lo = 0, hi = 0x7fffffff;  // the largest r known to hold too few, the least too many
   bool fits = false;
   for (int r = r_first;;) {
     const int x0 = max(0, ci - r), x1 = min(g.Gx - 1, ci + r);
     const int y0 = max(0, cj - r), y1 = min(g.Gy - 1, cj + r), rows = y1 - y0 + 1;
-    const bool all = x0 == 0 && x1 == g.Gx - 1 && y0 == 0 && y1 == g.Gy - 1;
+    const bool all_x = x0 == 0 && x1 == g.Gx - 1, all_y = y0 == 0 && y1 == g.Gy - 1;
+    const bool all = all_x && all_y;
     if (rows > 32) break;
     int s = 0, c = 0;
     if (lane < rows) {
@@ -223,8 +242,7 @@ __global__ void __launch_bounds__(128) k_knn_warp(
     sa[w][lane] = s - (pre - c);
     __syncwarp();
     int row = 0;
-    const double clear = (double)r * cmin * (1.0 - 1e-9);
-    const double lim = all ? __longlong_as_double(0x7ff0000000000000ll) : __dmul_rn(clear, clear);
+    const double lim = clearance2(g, r, all_x, all_y);
     kept = 0;
     for (int t0 = 0; t0 < M; t0 += 32) {
       const int t = t0 + lane;
@@ -249,19 +267,18 @@ __global__ void __launch_bounds__(128) k_knn_warp(
       kept += __popc(b);
     }
     __syncwarp();
-    if (kept > KNN_CAP) {  // too many: a smaller block, unless one was too small
-      if (r - 1 > lo) {
-        --r;
-        continue;
-      }
-      break;
-    }
-    if (kept >= K || all) {
+    if (kept <= KNN_CAP && (kept >= K || all)) {
       fits = true;
       break;
     }
-    lo = r;
-    ++r;
+    if (kept > KNN_CAP) hi = r;
+    else lo = r;
+    // the next block: between the two; a ring more while blocks are small (a
+    // square one stays below 32 rows of cells), then twice the rings, so that
+    // a long axis takes few steps
+    if (hi - lo <= 1) break;
+    const int up = lo < 16 ? lo + 1 : min(2 * lo, max(g.Gx, g.Gy));
+    r = hi == 0x7fffffff ? up : lo == 0 ? hi - 1 : lo + (hi - lo) / 2;
   }
   if (!fits) {
     if (lane == 0) rest[atomicAdd(nrest, 1)] = i;
@@ -351,17 +368,26 @@ __global__ void __launch_bounds__(128) k_knn_query(
   const double xi = x[i], yi = y[i];
   const bool bnd = tag != nullptr && tag[i] != 0;
   const int ci = cell_coord(xi, g.x0, g.ix, g.Gx), cj = cell_coord(yi, g.y0, g.iy, g.Gy);
-  const double cmin = fmin(g.cx, g.cy);
   double bd[KMAX];
   int bj[KMAX];
   int cnt = 0;
+  // offsets that exist along an axis: up to the grid's edges, or, periodic,
+  // the smallest offset of every column (row)
+  const int ymin = Ly > 0.0 ? -(g.Gy / 2) : -cj, ymax = Ly > 0.0 ? g.Gy / 2 : g.Gy - 1 - cj;
+  const int xmin = Lx > 0.0 ? -(g.Gx / 2) : -ci, xmax = Lx > 0.0 ? g.Gx / 2 : g.Gx - 1 - ci;
   for (int r = 0;; ++r) {
-    for (int dy = -r; dy <= r; ++dy) {
+    const bool ends = -r >= xmin || r <= xmax;
+    for (int dy = max(-r, ymin); dy <= min(r, ymax); ++dy) {
+      // the ring's first and last rows whole, of the others the two ends
+      const bool edge = (dy == -r || dy == r);
+      if (!edge && !ends) {
+        dy = r - 1;
+        continue;
+      }
       const int yy = ring_index(cj, dy, g.Gy, Ly > 0.0);
       if (yy < 0) continue;
-      const bool edge = (dy == -r || dy == r);
       const int stp = edge ? 1 : 2 * r;
-      for (int dx = -r; dx <= r; dx += stp) {
+      for (int dx = edge ? max(-r, xmin) : -r; dx <= (edge ? min(r, xmax) : r); dx += stp) {
         const int xx = ring_index(ci, dx, g.Gx, Lx > 0.0);
         if (xx < 0) continue;
         int c = yy * g.Gx + xx;
@@ -390,11 +416,9 @@ __global__ void __launch_bounds__(128) k_knn_query(
         }
       }
     }
-    if (cnt == K) {
-      double clear = (double)r * cmin * (1.0 - 1e-9);
-      if (bd[K - 1] < clear * clear) break;
-    }
-    if (r > max(g.Gx, g.Gy)) break;  // every cell visited
+    const bool all_x = -r <= xmin && r >= xmax, all_y = -r <= ymin && r >= ymax;
+    if (all_x && all_y) break;  // every cell visited
+    if (cnt == K && bd[K - 1] < clearance2(g, r, all_x, all_y)) break;
   }
   if (cnt < K) {
     atomicExch(err, 1);

@@ -1,5 +1,7 @@
 """The cloud search at the shapes where its cell grid and shared-memory lists
 can go wrong, bit-exact against the oracle's brute force."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -53,3 +55,51 @@ def test_graded_cloud_matches_brute_force():
     idx = torch.zeros((fp.n, 20), dtype=torch.int32, device="cuda:0")
     rbffd.rbffd_build_stencils(ctx(), dev(fp.x), dev(fp.y), dev(fp.tag), 20, idx)
     assert np.array_equal(idx.cpu().numpy(), oracle.knn(fp.x, fp.y, 20, fp.tag))
+
+
+def noisy_line(n, noise, seed):
+    r = np.random.Generator(np.random.PCG64(seed))
+    return np.sort(r.uniform(0, 1, n)), noise * r.uniform(-1, 1, n)
+
+
+def two_lines(seed):  # clusters far apart: most cells of the long axis are empty
+    x, y = noisy_line(1500, 1e-15, seed)
+    x[1400:] = 3.0 + 1000.0 * x[1400:]
+    return x, y
+
+
+LONG = {"noise_1e-15": lambda s: noisy_line(3000, 1e-15, s),
+        "noise_1e-6": lambda s: noisy_line(3000, 1e-6, s),
+        "noise_1e-3": lambda s: noisy_line(3000, 1e-3, s), "two_lines": two_lines}
+
+
+@pytest.mark.parametrize("q", [2, 20, 129])
+@pytest.mark.parametrize("upright", [False, True])
+@pytest.mark.parametrize("case", sorted(LONG))
+def test_boxes_longer_than_the_grid_match_brute_force(case, upright, q):
+    """Aspects beyond what square cells can follow: one column or row of cells
+    whose short side is far below the spacing."""
+    x, y = LONG[case](5)
+    if upright:
+        x, y = y, x
+    r = np.random.Generator(np.random.PCG64(q))
+    for tag in (None, (r.uniform(size=x.size) < 0.2).astype(np.int8)):
+        idx = torch.zeros((x.size, q), dtype=torch.int32, device="cuda:0")
+        rbffd.rbffd_build_stencils(ctx(), dev(x), dev(y), None if tag is None else dev(tag), q, idx)
+        assert np.array_equal(idx.cpu().numpy(), oracle.knn(x, y, q, tag)), (case, q, tag is None)
+
+
+def test_a_long_line_takes_no_longer_than_a_square_cloud():
+    """40 000 points on a line up to rounding: the search's work is that of
+    40 000 points (ring by ring along the line it would be 10 000 times that)."""
+    def seconds(x, y):
+        idx = torch.zeros((x.size, 20), dtype=torch.int32, device="cuda:0")
+        a = dev(np.ascontiguousarray(x)), dev(np.ascontiguousarray(y))
+        rbffd.rbffd_build_stencils(ctx(), *a, None, 20, idx)
+        t = time.perf_counter()
+        rbffd.rbffd_build_stencils(ctx(), *a, None, 20, idx)
+        return time.perf_counter() - t
+
+    square = seconds(*clouds.random_cloud(40000, 3))
+    for x, y in (noisy_line(40000, 1e-15, 3), noisy_line(40000, 1e-15, 3)[::-1]):
+        assert seconds(x, y) < 20 * square + 0.01
