@@ -22,30 +22,13 @@
 // this solve: cavity 99^2 (q = 20, multigrid) 7.0 -> 4.1 ms, Kovasznay 30^2
 // (Jacobi, one cluster) 12.8 -> 4.8 ms; four requests of 5 184 to 8 836 rows
 // served together, two time steps each, batched: 500 -> 372 ms.
+#include "bicg_scalars.cuh"
 #include "krylov.cuh"
 #include "resident.cuh"
 
 namespace rbffd {
 
 namespace {
-
-// As in krylov.cu: residual growth over the best that counts as a blow-up,
-// restarts from the best iterate, restarts after a breakdown.
-constexpr double BLOWUP2 = 1e20;  // squared
-constexpr int MAX_BLOWUPS = 8, MAX_BREAKDOWNS = 3;
-// A solve of CHECK_ITS iterations or more whose recurrence meets the tolerance
-// is checked against its true residual, and restarted from there where that
-// is over CHECK2^(1/2) times the tolerance, at most MAX_CHECKS times: after
-// thousands of iterations the two part (a 19 920-row channel, 7 257 Jacobi
-// iterations to 1e-12: fields 1.4e-8 off, against 4e-11 with a restart).
-constexpr double CHECK2 = 100.0;
-constexpr int MAX_CHECKS = 3, CHECK_ITS = 1000;
-
-struct Scalars {
-  double bnorm, tol2, rho, alpha, omega, beta, rr, best2, relres;
-  int it, restarts, blowups, state, need_init, restore, save, run, first, half;
-  int checks, met;  // true-residual checks made; the recurrence met the tolerance
-};
 
 struct BicgResArgs {
   KrylovArgs k;
@@ -80,7 +63,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
   using V = res::Vec<double, NR>;
   constexpr int VA = 3 * NR, VC = 5 * NR;
   __shared__ double wsum[VC * 32], cpart[2 * VC * RES_CLUSTER], tot[VC];
-  __shared__ Scalars ks[NR];
+  __shared__ BicgScalars ks[NR];
   __shared__ int s_any;
   extern __shared__ __align__(16) unsigned char dyn[];
   const KrylovArgs &K = A.k;
@@ -178,15 +161,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
       for (int e = tid; e < (k1 - k0) * A.ldb; e += RES_NT)
         Bs[e] = __ldg(A.B + (size_t)k0 * A.ldb + e);
   }
-  if (tid < NR) {
-    Scalars &c = ks[tid];
-    c.bnorm = c.rho = c.alpha = c.omega = 1.0;
-    c.beta = c.relres = c.rr = c.tol2 = 0.0;
-    c.best2 = 1e308;
-    c.it = c.restarts = c.blowups = c.restore = c.save = c.half = c.checks = c.met = 0;
-    c.state = KRY_RUNNING;
-    c.need_init = c.first = c.run = 1;
-  }
+  if (tid < NR) bicg_start(ks[tid]);
   for (int e = tid; e < nr; e += RES_NT)
 #pragma unroll
     for (int k = 0; k < NR; ++k) xo[e].x[k] = K.x[k][r0 + e];
@@ -334,26 +309,6 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
     return res::team_barrier(team);
   };
 
-  // the recurrence has met the tolerance (thread k)
-  auto met = [&](Scalars &c) {
-    if (c.checks >= MAX_CHECKS || c.it < CHECK_ITS) {
-      c.state = KRY_OK;
-    } else {
-      c.checks++;
-      c.met = c.need_init = 1;
-    }
-  };
-  // a system whose recurrence ran away (or became non-finite) restarts from
-  // its best iterate, a bounded number of times (thread k)
-  auto blowup = [&](Scalars &c, int final_state) {
-    if (c.blowups >= MAX_BLOWUPS || c.it >= K.maxit) {
-      c.state = final_state;
-    } else {
-      c.blowups++;
-      c.restore = c.need_init = 1;
-    }
-  };
-
   for (;;) {
     // ---------------- (re)starts: r = b - A x, r^ = p = r
     bool ini[NR], any_ini = false;
@@ -367,7 +322,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
 #pragma unroll
         for (int k = 0; k < NR; ++k)
           if (ini[k]) {
-            if (ks[k].restore) xo[e].x[k] = K.w[k].xb[r0 + e];
+            if (bicg_from_copy(ks[k])) xo[e].x[k] = K.w[k].xb[r0 + e];
             K.x[k][r0 + e] = xo[e].x[k];
           }
       if (!res::team_barrier(team)) { ok = false; break; }
@@ -396,40 +351,8 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
       }
       ok = res::team_totals<2 * NR, VC>(team, acc, tot, wsum, cpart, K.res.part, active);
       if (!ok) break;
-      if (tid < NR && ks[tid].state == KRY_RUNNING && ks[tid].need_init) {
-        Scalars &c = ks[tid];
-        c.need_init = c.restore = 0;
-        const double bb = tot[2 * tid], rr = tot[2 * tid + 1];
-        if (c.it == 0 && c.restarts == 0 && c.blowups == 0) {
-          c.bnorm = sqrt(bb);
-          c.tol2 = K.tol * K.tol * bb;
-        }
-        c.first = 1;
-        if (c.met) {
-          c.met = 0;
-          c.best2 = 1e308;
-          // the recurrence's residual is reported, as without the check
-          if (rr <= CHECK2 * c.tol2) c.state = KRY_OK;
-        }
-        if (c.state == KRY_RUNNING) c.rr = rr;
-        if (c.state == KRY_OK) {
-        } else if (c.bnorm == 0.0) {
-          c.rr = 0.0;
-          c.state = KRY_OK;
-          c.half = 3;  // x = 0
-        } else if (!(rr == rr)) {
-          c.state = KRY_DIVERGED;
-        } else if (rr <= c.tol2) {
-          c.state = KRY_OK;
-        } else {
-          if (rr < c.best2) {
-            c.best2 = rr;
-            c.save = 1;
-          }
-          c.rho = rr;
-          if (rr == 0.0) c.state = KRY_NOCONV;
-        }
-      }
+      if (tid < NR && ks[tid].state == KRY_RUNNING && ks[tid].need_init)
+        bicg_restarted(ks[tid], tot[2 * tid], tot[2 * tid + 1], K.tol);
       __syncthreads();
 #pragma unroll
       for (int k = 0; k < NR; ++k)
@@ -531,54 +454,8 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
       ok = res::team_totals<VA, VC>(team, acc, tot, wsum, cpart, K.res.part, active);
     }
     if (!ok) break;
-    if (tid < NR && ks[tid].run) {
-      Scalars &c = ks[tid];
-      const double rhv = tot[3 * tid], rr = tot[3 * tid + 1], rhr = tot[3 * tid + 2];
-      const bool was_first = c.first != 0;
-      c.first = c.save = 0;
-      c.run = 0;
-      if (!was_first) {
-        // the tests of the iteration whose x and r were just formed
-        c.rr = rr;
-        if (!isfinite(rr)) {
-          blowup(c, KRY_DIVERGED);
-        } else if (rr <= c.tol2) {
-          met(c);
-        } else {
-          bool go = true;
-          if (rr < c.best2) {
-            c.best2 = rr;
-            c.save = 1;  // copied to xb before the next update of x
-          } else if (rr > BLOWUP2 * c.best2) {
-            blowup(c, KRY_NOCONV);
-            go = false;
-          }
-          if (go && (c.omega == 0.0 || c.rho == 0.0)) {
-            // breakdown: restart from the current x
-            if (c.restarts >= MAX_BREAKDOWNS) {
-              c.state = KRY_NOCONV;
-            } else {
-              c.restarts++;
-              c.need_init = 1;
-            }
-            go = false;
-          }
-          if (go && c.it >= K.maxit) {
-            c.state = KRY_NOCONV;
-            go = false;
-          }
-          if (go) {
-            // rho' came from two products that cancel; (r^, r) summed
-            // directly replaces it (krylov.cu)
-            c.rho = rhr;
-            c.run = 1;
-          }
-        }
-      } else {
-        c.run = 1;
-      }
-      if (c.run) c.alpha = c.rho / rhv;
-    }
+    if (tid < NR && ks[tid].run)
+      bicg_after_v(ks[tid], tot[3 * tid], tot[3 * tid + 1], tot[3 * tid + 2], K.maxit);
     __syncthreads();
     bool anyc = false;
 #pragma unroll
@@ -655,27 +532,9 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
       const double om0 = __shfl_sync(0xffffffffu, quo, lane & ~3);
       const double iom = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 1);
       const double ar = __shfl_sync(0xffffffffu, quo, (lane & ~3) + 2);
-      if (k < NR && o == 0) {
-        Scalars &c = ks[k];
-        c.half = 0;
-        if (c.run) {
-          const double ss = tot[5 * k], rhs = tot[5 * k + 3], rht = tot[5 * k + 4];
-          c.it++;
-          if (!isfinite(ss)) {
-            c.half = 2;  // non-finite s: restart from the best iterate
-            blowup(c, KRY_DIVERGED);
-          } else if (ss <= c.tol2) {
-            c.half = 1;
-            c.rr = ss;
-            met(c);
-          } else {
-            c.omega = tt == 0.0 ? 0.0 : om0;
-            const double rho_new = rhs - c.omega * rht;
-            c.beta = (c.omega == 0.0 || c.rho == 0.0) ? 0.0 : rho_new * ar * iom;
-            c.rho = rho_new;
-          }
-        }
-      }
+      if (k < NR && o == 0)
+        bicg_after_t(ks[k], tot[5 * k], tot[5 * k + 3], tot[5 * k + 4], tt == 0.0, om0, iom, ar,
+                     K.maxit);
     }
     __syncthreads();
 #pragma unroll
@@ -694,7 +553,7 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
     for (int k = 0; k < NR; ++k) K.x[k][r0 + e] = xo[e].x[k];
   if (team.cluster) res::team_barrier(team);  // no CTA leaves while others may write to it
   if (lb == 0 && tid < NR) {
-    const Scalars &c = ks[tid];
+    const BicgScalars &c = ks[tid];
     K.out[tid].iters = c.it;
     K.out[tid].restarts = c.restarts + c.blowups;
     K.out[tid].status = ok ? c.state : KRY_TIMEOUT;
