@@ -17,7 +17,9 @@ constexpr int BICG_BLOWUPS = 8, BICG_BREAKDOWNS = 3;
 // where that is over BICG_CHECK2^(1/2) times the tolerance, at most BICG_CHECKS
 // times: after thousands of iterations the two part (a 19 920-row channel,
 // 7 257 Jacobi iterations to 1e-12: fields 1.4e-8 off, against 4e-11 with a
-// restart).
+// restart).  The check refines a solve that has met its tolerance: where the
+// restart does not meet it again (no iterations left, a breakdown), the solve
+// ends as met, with the best iterate since (bicg_end).
 constexpr double BICG_CHECK2 = 100.0;
 constexpr int BICG_CHECKS = 3, BICG_CHECK_ITS = 1000;
 
@@ -29,6 +31,8 @@ struct BicgScalars {
   int save;       // x is the best iterate, to be copied before it is updated
   int run, first, half;
   int checks, met;  // true-residual checks made; the recurrence met the tolerance
+  int held;         // a checked iterate of finite residual is there to fall back on
+  double met_rr;    // (r, r) of the recurrence when it last met the tolerance
 };
 
 // A system whose recurrence ran away (or became non-finite) restarts from its
@@ -49,14 +53,15 @@ __host__ __device__ inline void bicg_met(BicgScalars &c) {
   } else {
     c.checks++;
     c.met = c.need_init = 1;
+    c.met_rr = c.rr;
   }
 }
 
 __host__ __device__ inline void bicg_start(BicgScalars &c) {
   c.bnorm = c.rho = c.alpha = c.omega = 1.0;
-  c.beta = c.rr = c.tol2 = 0.0;
+  c.beta = c.rr = c.tol2 = c.met_rr = 0.0;
   c.best2 = 1e308;
-  c.it = c.restarts = c.blowups = c.restore = c.save = c.half = c.checks = c.met = 0;
+  c.it = c.restarts = c.blowups = c.restore = c.save = c.half = c.checks = c.met = c.held = 0;
   c.state = KRY_RUNNING;
   c.need_init = c.first = c.run = 1;
 }
@@ -81,6 +86,7 @@ __host__ __device__ inline void bicg_restarted(BicgScalars &c, double bb, double
     c.best2 = 1e308;
     // the recurrence's residual is reported, as without the check
     if (rr <= BICG_CHECK2 * c.tol2) c.state = KRY_OK;
+    else c.held |= rr == rr;
   }
   if (c.state == KRY_RUNNING) c.rr = rr;
   if (c.state == KRY_OK) {
@@ -172,6 +178,16 @@ __host__ __device__ inline void bicg_after_t(BicgScalars &c, double ss, double r
     c.beta = (c.omega == 0.0 || c.rho == 0.0) ? 0.0 : rho_new * ar * iom;
     c.rho = rho_new;
   }
+}
+
+// The end of a solve: true when x has to be taken from the best iterate's copy.
+// A solve that met its tolerance and was restarted from the true residual does
+// not fail for what came after.
+__host__ __device__ inline bool bicg_end(BicgScalars &c) {
+  if (c.state == KRY_OK || c.state == KRY_RUNNING || !c.held) return false;
+  c.state = KRY_OK;
+  c.rr = c.met_rr;
+  return !c.save;
 }
 
 }  // namespace rbffd

@@ -548,9 +548,12 @@ __device__ __forceinline__ void bicg_res_body(const BicgResArgs &A, const int lb
     __syncthreads();
   }
   // ---- the solution (also of a solve that stopped short)
+  if (tid < NR && ok) ks[tid].half = bicg_end(ks[tid]) ? 4 : 0;
+  __syncthreads();
   for (int e = tid; e < nr; e += RES_NT)
 #pragma unroll
-    for (int k = 0; k < NR; ++k) K.x[k][r0 + e] = xo[e].x[k];
+    for (int k = 0; k < NR; ++k)
+      K.x[k][r0 + e] = ks[k].half == 4 ? K.w[k].xb[r0 + e] : xo[e].x[k];
   if (team.cluster) res::team_barrier(team);  // no CTA leaves while others may write to it
   if (lb == 0 && tid < NR) {
     const BicgScalars &c = ks[tid];

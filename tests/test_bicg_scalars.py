@@ -2,7 +2,9 @@
 the host: random solves whose residuals fall, blow up, break down and become
 non-finite in either phase, with the iterates as numbers.  The copy of the best
 iterate is the one whose residual the blow-up test compares with, and a restart
-from the best iterate starts from it."""
+from the best iterate starts from it.  A solve that met its tolerance, was found
+far from it by its true residual and went on ends as met, with an iterate no
+worse than the one it was checked at."""
 import os
 import subprocess
 
@@ -24,14 +26,16 @@ static double u01() {
 
 int main() {
   std::map<std::string, int> n;
-  const double inf = 1e308 * 10, tol = 1e-12;
+  const double inf = 1e308 * 10, tol = 1e-4;
   for (int solve = 0; solve < 20000; ++solve) {
     BicgScalars c;
     bicg_start(c);
-    const int maxit = 20 + (int)(180 * u01());
+    const bool is_long = solve % 2;  // long enough for the true-residual check
+    const int maxit = 20 + (int)(180 * u01()) + (is_long ? BICG_CHECK_ITS : 0);
     const double p_s = 0.05 * u01(), p_r = 0.05 * u01(), p_blow = 0.1 * u01(), p_zero = 0.02 * u01();
     std::map<int, double> res;  // squared residual of every iterate
     int x = 0, xb = -1, made = 0;
+    double checked = -1.0;  // largest true residual that a check found and went on from
     res[0] = 1.0;
     for (;;) {
       if (c.state == KRY_RUNNING && c.need_init) {
@@ -41,7 +45,15 @@ int main() {
           n["restores"]++;
           if (res[x] != c.best2) n["not_from_best"]++;
         }
+        if (c.met) {
+          n["checks"]++;
+          if (u01() < 0.7) {
+            res[x] *= 1e6;
+            if (res[x] > BICG_CHECK2 * c.tol2) checked = fmax(checked, res[x]);
+          }
+        }
         bicg_restarted(c, 1.0, res[x], tol);
+        if (is_long && c.it == 0) c.it = BICG_CHECK_ITS;
       }
       if (c.state != KRY_RUNNING) break;
       const bool first = c.first;
@@ -50,7 +62,7 @@ int main() {
       // the iterate just formed: falling, blown up, or no number
       double rr = res[first ? x : x - 1 < 0 ? 0 : x - 1];
       if (!first) {
-        rr *= u01() < 0.6 ? 0.5 : 1.6;
+        rr *= u01() < 0.6 ? (is_long ? 0.2 : 0.5) : 1.6;
         if (u01() < p_blow) rr *= 1e21;
         if (u01() < p_r) rr = inf;
         res[x] = rr;
@@ -66,10 +78,21 @@ int main() {
       if (c.half == 1) res[x = ++made] = ss;
     }
     if (c.state == KRY_RUNNING) n["unfinished"]++;
+    const int before = c.state;
+    if (bicg_end(c)) x = xb;
+    if (checked > 0.0) {
+      n["went_on"]++;
+      if (before != KRY_OK) n["kept"]++;
+      if (c.state != KRY_OK || c.rr > c.tol2) n["failed_after_met"]++;
+      if (!(res[x] <= checked)) n["worse_than_checked"]++;
+    } else if (c.state != before) {
+      n["changed_end"]++;
+    }
     n["solves"]++;
   }
   for (const char *k : {"solves", "restores", "non_finite_s", "unfinished", "not_from_best",
-                        "copy_not_best", "saves_not_best"})
+                        "copy_not_best", "saves_not_best", "checks", "went_on", "kept",
+                        "failed_after_met", "worse_than_checked", "changed_end"})
     printf("%s %d\n", k, n[k]);
 }
 """
@@ -92,3 +115,9 @@ def test_a_restart_starts_from_the_best_iterate(counts):
     assert counts["restores"] > 1000 and counts["non_finite_s"] > 1000
     assert counts["not_from_best"] == 0
     assert counts["copy_not_best"] == counts["saves_not_best"] == 0
+
+
+def test_a_solve_that_met_its_tolerance_does_not_fail_after_it(counts):
+    assert counts["checks"] > 1000 and counts["went_on"] > 500 and counts["kept"] > 100
+    assert counts["failed_after_met"] == counts["worse_than_checked"] == 0
+    assert counts["changed_end"] == 0
