@@ -112,7 +112,10 @@ typedef struct rbffd_problem rbffd_problem;
 /* ---------------------------------------------------------------- context */
 
 /* Create a context on CUDA device `device`.  hbm_budget_bytes caps what
- * problems of this context may allocate (0 = no cap).  cuda_stream is a
+ * problems of this context may allocate (0 = no cap).  Memory held for speed
+ * alone (a workspace kept between calls, the resident solves' lists and dense
+ * coarse operators) is given back before an allocation is refused; the solves
+ * of such problems then stream, and rbffd_problem_bytes falls.  cuda_stream is a
  * cudaStream_t to issue work on, or NULL for a stream owned by the context.
  * Errors: RBFFD_EINVAL (bad device), RBFFD_ECUDA. */
 int rbffd_ctx_create(rbffd_ctx **out, int device, size_t hbm_budget_bytes, void *cuda_stream);

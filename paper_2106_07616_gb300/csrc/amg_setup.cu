@@ -49,17 +49,19 @@ struct Scratch {
   int take(T **p, size_t n) {
     *p = nullptr;
     const size_t bytes = std::max<size_t>(1, n) * sizeof(T);
-    if (!dev_reserve(ctx, bytes)) return RBFFD_ENOMEM;
-    void *v = nullptr;
-    if (cudaMallocAsync(&v, bytes, st) != cudaSuccess) {
+    do {
+      if (!dev_reserve(ctx, bytes)) continue;
+      void *v = nullptr;
+      if (cudaMallocAsync(&v, bytes, st) == cudaSuccess) {
+        held.emplace_back(v, bytes);
+        *p = (T *)v;
+        return RBFFD_OK;
+      }
       cudaGetLastError();
       dev_release(ctx, bytes);
       set_error("multigrid setup: cudaMallocAsync(%zu) failed", bytes);
-      return RBFFD_ENOMEM;
-    }
-    held.emplace_back(v, bytes);
-    *p = (T *)v;
-    return RBFFD_OK;
+    } while (ctx_give_back(ctx, bytes));
+    return RBFFD_ENOMEM;
   }
   ~Scratch() {
     for (auto &h : held) {

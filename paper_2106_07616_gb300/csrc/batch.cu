@@ -87,7 +87,8 @@ int BatchScratch::reserve(rbffd_ctx *c, int members) {
     cudaFreeHost(hmem);
     hmem = nullptr;
   }
-  cap = std::max(members, 16);
+  cap = 0;  // until both buffers are there
+  const int want = std::max(members, 16);
   maxc = std::max({krylov_batch_max_ctas(ctx, 1), krylov_batch_max_ctas(ctx, 2),
                    fgmres_batch_max_ctas(ctx), krylov_ir_batch_max_ctas(ctx, 1, INNER_F32),
                    krylov_ir_batch_max_ctas(ctx, 2, INNER_F32),
@@ -103,20 +104,21 @@ int BatchScratch::reserve(rbffd_ctx *c, int members) {
   };
   for (int k = 0; k < NSLOT; ++k) {
     off_sys[k] = take(std::max({sizeof(KrylovArgs), sizeof(FgmresArgs), sizeof(MixedArgs),
-                                krylov_res_args_bytes()}) * cap);
+                                krylov_res_args_bytes()}) * want);
     off_cta_sys[k] = take(sizeof(int) * maxc);
-    team_words = 4 * maxc + cap;
+    team_words = 4 * maxc + want;
     off_cta_first[k] = take(sizeof(int) * team_words);
     off_flags[k] = take(sizeof(unsigned int) * maxc);
-    off_bars[k] = take(sizeof(GridBarrier) * cap);
+    off_bars[k] = take(sizeof(GridBarrier) * want);
   }
-  off_recs = take(sizeof(void *) * cap);
-  off_kouts = take(sizeof(void *) * cap);
-  off_out = take(sizeof(MemberOut) * cap);
+  off_recs = take(sizeof(void *) * want);
+  off_kouts = take(sizeof(void *) * want);
+  off_out = take(sizeof(MemberOut) * want);
   dbytes = o;
   RBFFD_TRY(dev_alloc(ctx, &dmem, dbytes));
   hbytes = dbytes;
   RBFFD_CK(cudaMallocHost(&hmem, hbytes));
+  cap = want;
   return RBFFD_OK;
 }
 

@@ -10,8 +10,11 @@
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
+#include <vector>
 
 #include "rbffd.h"
+
+struct rbffd_problem;
 
 struct rbffd_ctx {
   int device = 0;
@@ -38,6 +41,9 @@ struct rbffd_ctx {
   // (ctx_scratch), freed with the context
   void *scratch = nullptr;
   size_t scratch_bytes = 0;
+  // the problems alive on this context: what they hold for speed alone goes
+  // back when an allocation finds no memory (ctx_give_back)
+  std::vector<rbffd_problem *> problems;
   // pinned host scratch for small read-backs
   void *pinned = nullptr;
   size_t pinned_bytes = 0;
@@ -107,8 +113,18 @@ inline int after_launch(rbffd_ctx *ctx, const char *what) {
 void ctx_ref(rbffd_ctx *ctx);
 void ctx_unref(rbffd_ctx *ctx);
 
-// Device allocation charged to the context's budget.
+// Device allocation charged to the context's budget.  Where it finds no memory,
+// what the context holds for speed alone is given back first; dev_try_alloc,
+// for such things themselves, fails instead.
 int dev_alloc(rbffd_ctx *ctx, void **p, size_t bytes);
+int dev_try_alloc(rbffd_ctx *ctx, void **p, size_t bytes);
+// Give back one kind of what the context holds for speed alone -- the kept
+// workspace, then the problems' dense coarse operators, then their resident
+// lists (their solves then stream) -- when `bytes` more cannot be had: true if
+// something was freed.  Nothing is freed where the budget would not hold
+// `bytes` even without all of it.  Waits for the context's stream; not
+// between the choice of a launch's arguments and the launch.
+bool ctx_give_back(rbffd_ctx *ctx, size_t bytes);
 void dev_free(rbffd_ctx *ctx, void *p, size_t bytes);
 // count `bytes` against the context's budget (false: it would exceed it;
 // the error text is set) / give them back
@@ -118,6 +134,7 @@ void dev_release(rbffd_ctx *ctx, size_t bytes);
 // context (its calls are serialised, and each waits for its own kernels).
 // Kept between calls -- cudaMalloc and cudaFree cost 0.1 ms and more a call --
 // up to 64 MB; a larger one replaces it and is given back at the next call.
+// No allocation may be made while it is in use.
 int ctx_scratch(rbffd_ctx *ctx, size_t bytes, void **out);
 void ctx_scratch_free(rbffd_ctx *ctx);
 // Small pinned host buffer of at least `bytes` (owned by the context).

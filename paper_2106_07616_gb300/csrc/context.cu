@@ -31,6 +31,13 @@ bool dev_reserve(rbffd_ctx *ctx, size_t bytes) {
 void dev_release(rbffd_ctx *ctx, size_t bytes) { ctx->used.fetch_sub(bytes); }
 
 int dev_alloc(rbffd_ctx *ctx, void **p, size_t bytes) {
+  for (;;) {
+    const int rc = dev_try_alloc(ctx, p, bytes);
+    if (rc != RBFFD_ENOMEM || !ctx_give_back(ctx, bytes)) return rc;
+  }
+}
+
+int dev_try_alloc(rbffd_ctx *ctx, void **p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return RBFFD_OK;
   if (!dev_reserve(ctx, bytes)) return RBFFD_ENOMEM;

@@ -1,5 +1,6 @@
 // problem.cu -- problem lifetime and the outer-iteration / time-step /
 // steady and unsteady drivers (paper Sec. 3.2), behind the C ABI.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -74,6 +75,46 @@ int check_desc(const rbffd_problem_desc *d) {
   return RBFFD_OK;
 }
 
+// Counts the builds of all problems, and what else makes a captured batched
+// iteration of a problem stale (batch.cu: graph_key).
+std::atomic<uint64_t> generation{0};
+
+void free_dense(rbffd_problem *P) {
+  if (P->fgB || P->amgB) dev_free(P->ctx, P->fgB ? (void *)P->fgB : P->amgB, P->fgB_bytes);
+  P->fgB = nullptr;
+  P->amgB = nullptr;
+  P->fgB_bytes = 0;
+}
+
+void free_lists(rbffd_problem *P) {
+  dev_free(P->ctx, P->res_mem, P->res_bytes);
+  P->res_mem = nullptr;
+  P->res_bytes = 0;
+  P->res = ResPlan();
+  P->res_hm_known = false;
+  memset(P->res_hm, 0, sizeof(P->res_hm));
+}
+
+// Team and room for the lists of the resident solves, unless they are there;
+// without memory for them the solves stream.
+void take_lists(rbffd_problem *P) {
+  if (P->res_mem) return;
+  ResPlan p = res_plan(P->ctx, P->n, P->q);
+  if (p.nb < 1) return;
+  Carver c;
+  const size_t o_hl = c.take<int32_t>((size_t)p.nb * p.hstride),
+               o_hi = c.take<int32_t>(2 * (size_t)p.nb),
+               o_li = c.take<uint16_t>((size_t)P->ldn * P->q), o_rp = c.take<char>(RES_PART_BYTES);
+  if (dev_try_alloc(P->ctx, &P->res_mem, c.off) != RBFFD_OK) return;
+  P->res_bytes = c.off;
+  char *b = (char *)P->res_mem;
+  p.hlist = P->res_hlist = (int32_t *)(b + o_hl);
+  p.hinfo = P->res_hinfo = (int32_t *)(b + o_hi);
+  p.lidx = P->res_lidx = (uint16_t *)(b + o_li);
+  p.part = b + o_rp;
+  P->res = p;
+}
+
 void free_amg(rbffd_problem *P) {
   if (P->amg_job) amg_build_abandon(P->amg_job);
   P->amg_job = nullptr;
@@ -85,10 +126,7 @@ void free_amg(rbffd_problem *P) {
   P->fg_mem = nullptr;
   P->fg_bytes = 0;
   P->fgV = P->fgZ = nullptr;
-  if (P->fgB || P->amgB) dev_free(P->ctx, P->fgB ? (void *)P->fgB : P->amgB, P->fgB_bytes);
-  P->fgB = nullptr;
-  P->amgB = nullptr;
-  P->fgB_bytes = 0;
+  free_dense(P);
   P->fgR = nullptr;
   P->fgpart = nullptr;
   P->amgf = nullptr;
@@ -102,7 +140,6 @@ void free_amg(rbffd_problem *P) {
 
 // Copy the inputs, build clouds, weights and operators, reset the state.
 int build(rbffd_problem *P, const rbffd_problem_desc *d) {
-  static std::atomic<uint64_t> generation{0};
   P->gen = ++generation;
   rbffd_ctx *ctx = P->ctx;
   cudaStream_t st = ctx->stream;
@@ -114,6 +151,7 @@ int build(rbffd_problem *P, const rbffd_problem_desc *d) {
   P->amg_err = RBFFD_OK;
   P->amg_errmsg[0] = 0;
   P->z_ready = false;
+  take_lists(P);
   // the compatible shift starts again from zero with the new operators
   RBFFD_CK(cudaMemsetAsync(&P->rec->cshift, 0, sizeof(double), ctx->stream));
   const size_t nb = (size_t)d->n * sizeof(double);
@@ -250,6 +288,28 @@ int krylov_status_code(int s) {
 
 }  // namespace
 
+bool rbffd::ctx_give_back(rbffd_ctx *ctx, size_t bytes) {
+  size_t dense = 0, lists = 0;
+  for (const rbffd_problem *P : ctx->problems) {
+    dense += P->fgB_bytes;
+    lists += P->res_bytes;
+  }
+  const size_t all = ctx->scratch_bytes + dense + lists;
+  if (all == 0 || (ctx->budget && ctx->used.load() - all + bytes > ctx->budget)) return false;
+  if (ctx->scratch) {
+    ctx_scratch_free(ctx);
+    return true;
+  }
+  cudaStreamSynchronize(ctx->stream);
+  for (rbffd_problem *P : ctx->problems) {
+    if (dense == 0 ? P->res_bytes == 0 : P->fgB_bytes == 0) continue;
+    P->gen = ++generation;
+    if (dense > 0) free_dense(P);
+    else free_lists(P);
+  }
+  return true;
+}
+
 int rbffd::amg_ready(rbffd_problem *P) {
   if (P->amg_err != RBFFD_OK) {  // the build failed for good: say so every time
     set_error("%s", P->amg_errmsg);
@@ -330,7 +390,7 @@ int issue_pcorr(rbffd_problem *P, double tol, int maxit, double inner_tol, int i
     // the composed cycle's phases
     const int ld = P->res.nb > 0 && !P->fgB ? fgmres_dense_ld(P->amgf_host) : 0;
     const size_t bytes = sizeof(float) * (size_t)ld * (ld > 0 ? P->amgf_host.lev[1].n : 0);
-    if (ld > 0 && dev_alloc(ctx, (void **)&P->fgB, bytes) == RBFFD_OK) {
+    if (ld > 0 && dev_try_alloc(ctx, (void **)&P->fgB, bytes) == RBFFD_OK) {
       P->fgB_bytes = bytes;
       RBFFD_TRY(fgmres_dense_build(ctx, P->amgf_host, P->fgB));
     }
@@ -617,7 +677,7 @@ int rbffd::team_sizes_ready(rbffd_problem *const *P, int m) {
 int rbffd::dense64_ready(rbffd_problem *P) {
   const int ld = P->amg && P->res.nb > 0 && !P->amgB ? krylov_dense_ld(P->amg_host) : 0;
   const size_t bytes = sizeof(double) * (size_t)ld * ld;
-  if (ld > 0 && dev_alloc(P->ctx, (void **)&P->amgB, bytes) == RBFFD_OK) {
+  if (ld > 0 && dev_try_alloc(P->ctx, (void **)&P->amgB, bytes) == RBFFD_OK) {
     P->fgB_bytes = bytes;
     RBFFD_TRY(krylov_dense_build(P->ctx, P->amg_host, P->amgB));
   }
@@ -678,7 +738,6 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       if (P->kblocks2 > c2) P->kblocks2 = c2;
     }
     P->rblocks = ops_reduce_blocks(ctx, n);
-    P->res = res_plan(ctx, n);
     // partials: room for two right-hand sides over the larger grid (a batched
     // launch may give one member two single-RHS systems, or one system twice
     // the CTAs)
@@ -719,38 +778,15 @@ extern "C" int rbffd_problem_create(rbffd_ctx *ctx, const rbffd_problem_desc *d,
       o_part64 = c.take<double>(krylov_ir_partials64(2, kb));
       o_part32 = c.take<char>(krylov_ir_partials_inner_bytes(2, kb, P->inner));
     }
-    size_t o_hl = 0, o_hi = 0, o_li = 0, o_rp = 0;
-    const size_t streaming = c.off;
-    if (P->res.nb > 0) {
-      o_hl = c.take<int32_t>((size_t)P->res.nb * P->res.hstride);
-      o_hi = c.take<int32_t>(2 * (size_t)P->res.nb);
-      o_li = c.take<uint16_t>(lq);
-      o_rp = c.take<char>(RES_PART_BYTES);
-    }
     P->bytes = c.off;
     int rc = dev_alloc(ctx, &P->mem, P->bytes);
-    if (rc == RBFFD_ENOMEM) {
-      // the context's own workspace goes first, then the resident solves
-      ctx_scratch_free(ctx);
-      rc = dev_alloc(ctx, &P->mem, P->bytes);
-    }
-    if (rc == RBFFD_ENOMEM && P->res.nb > 0) {
-      P->res = ResPlan();
-      P->bytes = streaming;
-      rc = dev_alloc(ctx, &P->mem, P->bytes);
-    }
     if (rc != RBFFD_OK) {
       delete P;
       ctx_unref(ctx);
       return rc;
     }
+    ctx->problems.push_back(P);
     char *b = (char *)P->mem;
-    if (P->res.nb > 0) {
-      P->res.hlist = P->res_hlist = (int32_t *)(b + o_hl);
-      P->res.hinfo = P->res_hinfo = (int32_t *)(b + o_hi);
-      P->res.lidx = P->res_lidx = (uint16_t *)(b + o_li);
-      P->res.part = b + o_rp;
-    }
     P->x = (double *)(b + o_x);
     P->y = (double *)(b + o_y);
     P->nx = (double *)(b + o_nx);
@@ -837,13 +873,16 @@ extern "C" void rbffd_problem_destroy(rbffd_problem *P) {
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
   free_amg(P);
+  free_lists(P);
   dev_free(ctx, P->mem, P->bytes);
+  ctx->problems.erase(std::find(ctx->problems.begin(), ctx->problems.end(), P));
   delete P;
   ctx_unref(ctx);
 }
 
 extern "C" size_t rbffd_problem_bytes(const rbffd_problem *P) {
-  return P ? P->bytes + P->amg_bytes + P->amg0_bytes + P->fg_bytes + P->fgB_bytes : 0;
+  return P ? P->bytes + P->res_bytes + P->amg_bytes + P->amg0_bytes + P->fg_bytes + P->fgB_bytes
+           : 0;
 }
 
 static void report_levels(const AmgInfo &I, bool have_any, int32_t *levels, int32_t *rows,

@@ -48,9 +48,12 @@ struct rbffd_problem {
   rbffd::MixedVecs mv[2] = {};
   double *part64 = nullptr;
   void *partin = nullptr;
-  // team and halo lists of the resident solves (nb = 0: none); its arrays
-  // are in this allocation, rebuilt with the clouds
+  // team and halo lists of the resident solves (nb = 0: none), rebuilt with
+  // the clouds; in an allocation of their own, which goes back when the
+  // context runs out of memory
   rbffd::ResPlan res;
+  void *res_mem = nullptr;
+  size_t res_bytes = 0;
   int32_t *res_hlist = nullptr, *res_hinfo = nullptr;
   uint16_t *res_lidx = nullptr;
   // longest halo list at each team size of a batched resident solve (0: none)

@@ -2,6 +2,8 @@
 // (resident.cuh), made once per build of a problem.
 #include "resident.cuh"
 
+#include <algorithm>
+
 #include "krylov.cuh"
 
 namespace rbffd {
@@ -113,7 +115,7 @@ int res_halo_sizes(rbffd_ctx *ctx, int n, int q, int ldn, const int32_t *col, in
   return after_launch(ctx, "k_halo_sizes");
 }
 
-ResPlan res_plan(rbffd_ctx *ctx, int n) {
+ResPlan res_plan(rbffd_ctx *ctx, int n, int q) {
   ResPlan p;
   const int cap = ctx->num_sms < RES_MAXB ? ctx->num_sms : RES_MAXB;
   // eight lanes a row before the rows spread over fewer SMs
@@ -128,7 +130,8 @@ ResPlan res_plan(rbffd_ctx *ctx, int n) {
   p.R = (n + nb - 1) / nb;
   for (int t = 2; t <= 8; ++t)
     if ((32 / t) * (RES_NT / 32) >= p.R) p.T = t;
-  p.hstride = n < RES_HCAP ? n : RES_HCAP;
+  // no list is longer than the cloud, or than its rows' entries
+  p.hstride = (int)std::min({(long long)n, (long long)RES_HCAP, (long long)p.R * q});
   return p;
 }
 

@@ -76,7 +76,7 @@ int res_halo_sizes(rbffd_ctx *ctx, int n, int q, int ldn, const int32_t *col, in
 
 // Rows and lanes of a team for n rows (nb = 0 when a CTA would own more rows
 // than it has threads).
-ResPlan res_plan(rbffd_ctx *ctx, int n);
+ResPlan res_plan(rbffd_ctx *ctx, int n, int q);
 // Lists of a packed matrix's columns; longest list to *d_hmax (device).
 int res_halo_build(rbffd_ctx *ctx, const ResPlan &p, int n, int q, int ldn, const int32_t *col,
                    int32_t *hlist, int32_t *hinfo, uint16_t *lidx, int *d_hmax);
