@@ -622,10 +622,9 @@ static int launch_resident(BatchScratch &S, int slot, int nr, const std::vector<
   RBFFD_TRY(put_tables(S, slot, T, m, bytes));
   RBFFD_CK(cudaMemsetAsync(dflags, 0, sizeof(unsigned int) * m, ctx->stream));
   RBFFD_TRY(reset_barriers(ctx, dbars, m));
-  *ran = true;
   return krylov_res_batch_launch(ctx, nr, amg, T.nctas, db + S.off_sys[slot],
                                  (const int *)(db + S.off_cta_sys[slot]),
-                                 (const int *)(db + S.off_cta_first[slot]), smem);
+                                 (const int *)(db + S.off_cta_first[slot]), smem, ran);
 }
 
 // One batched Krylov launch for the systems args[0..m) (args filled except

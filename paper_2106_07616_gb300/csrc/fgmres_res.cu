@@ -671,8 +671,8 @@ int fgmres_res_launch(rbffd_ctx *ctx, const FgmresArgs &args, const ResPlan &res
   RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
   if (!res.cluster)
     RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
-  *ran = true;
-  return res_launch(ctx, res, fn, &a, smem, "k_fgmres_res");
+  *ran = res_launch(ctx, res, fn, &a, smem);
+  return RBFFD_OK;
 }
 
 }  // namespace rbffd

@@ -116,7 +116,7 @@ size_t krylov_res_args_bytes();
 bool krylov_res_args(int nr, const KrylovArgs &args, const AmgDev *h, double omega,
                      const double *B, void *out, size_t *smem);
 int krylov_res_batch_launch(rbffd_ctx *ctx, int nr, bool amg, int nctas, const void *d_sys,
-                            const int *d_cta_team, const int *d_info, size_t smem);
+                            const int *d_cta_team, const int *d_info, size_t smem, bool *ran);
 int krylov_dense_ld(const AmgDev &h);
 int krylov_dense_build(rbffd_ctx *ctx, const AmgDev &h, double *B);
 size_t krylov_partials_doubles(int nr, int nblocks);

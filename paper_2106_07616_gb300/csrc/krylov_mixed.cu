@@ -1111,14 +1111,15 @@ const void *ir_res_kernel(int nr, int inner, bool ff_sums, int q, const ResPlan 
 static int ir_res_launch(rbffd_ctx *ctx, int nr, const MixedArgs &args, bool *ran) {
   size_t smem = 0;
   const void *fn = ir_res_kernel(nr, args.inner, args.ff_sums != 0, args.q, args.res, &smem);
-  *ran = fn != nullptr;
+  *ran = false;
   if (!fn) return RBFFD_OK;
   MixedArgs a = args;
   a.tpr = args.res.T;
   a.o_xold = (int)ir_res_halo_bytes(args.inner == INNER_FF ? 8 : 4, nr, args.res);
   RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
   if (!args.res.cluster) RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
-  return res_launch(ctx, args.res, fn, &a, smem, "k_ir_res");
+  *ran = res_launch(ctx, args.res, fn, &a, smem);
+  return RBFFD_OK;
 }
 
 // Batched launch: system cta_sys[b] owns the consecutive CTAs from

@@ -714,11 +714,11 @@ int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgD
   if (!res_args(nr, args, h, omega, B, &a, &smem)) return RBFFD_OK;
   RBFFD_TRY(reset_barriers(ctx, args.bar, 1));
   if (!p.cluster) RBFFD_CK(cudaMemsetAsync(args.flags, 0, sizeof(unsigned int), ctx->stream));
-  *ran = true;
   const void *fn = amg       ? (const void *)k_bicg_res<1, true>
                    : nr == 1 ? (const void *)k_bicg_res<1, false>
                              : (const void *)k_bicg_res<2, false>;
-  return res_launch(ctx, p, fn, &a, smem, "k_bicg_res");
+  *ran = res_launch(ctx, p, fn, &a, smem);
+  return RBFFD_OK;
 }
 
 size_t krylov_res_args_bytes() { return sizeof(BicgResArgs); }
@@ -733,19 +733,17 @@ bool krylov_res_args(int nr, const KrylovArgs &args, const AmgDev *h, double ome
 }
 
 int krylov_res_batch_launch(rbffd_ctx *ctx, int nr, bool amg, int nctas, const void *d_sys,
-                            const int *d_cta_team, const int *d_info, size_t smem) {
+                            const int *d_cta_team, const int *d_info, size_t smem, bool *ran) {
   const void *fn = amg       ? (const void *)k_bicg_res_batch<1, true>
                    : nr == 1 ? (const void *)k_bicg_res_batch<1, false>
                              : (const void *)k_bicg_res_batch<2, false>;
-  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
   void *kargs[] = {(void *)&d_sys, (void *)&d_cta_team, (void *)&d_info};
-  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nctas), dim3(RES_NT), kargs, smem,
-                                                    ctx->stream);
-  ctx->launches++;
-  if (e != cudaSuccess) {
-    set_error("cooperative launch of k_bicg_res_batch failed: %s", cudaGetErrorString(e));
-    return RBFFD_ECUDA;
-  }
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM);
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel(fn, dim3(nctas), dim3(RES_NT), kargs, smem, ctx->stream);
+  *ran = e == cudaSuccess;  // refused: as res_launch
+  if (*ran) ctx->launches++;
+  else cudaGetLastError();
   return RBFFD_OK;
 }
 

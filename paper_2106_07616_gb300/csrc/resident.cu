@@ -146,18 +146,17 @@ int res_halo_build(rbffd_ctx *ctx, const ResPlan &p, int n, int q, int ldn, cons
   return after_launch(ctx, "k_halo_build");
 }
 
-int res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, size_t smem,
-               const char *what) {
-  RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
+bool res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nb);
   cfg.blockDim = dim3(RES_NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = ctx->stream;
   cudaLaunchAttribute at[1];
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM);
   if (p.cluster) {
-    if (p.nb > 8)
-      RBFFD_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (e == cudaSuccess && p.nb > 8)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = p.nb;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
@@ -168,14 +167,13 @@ int res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, siz
   cfg.attrs = at;
   cfg.numAttrs = 1;
   void *kargs[] = {args};
-  const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, kargs);
-  ctx->launches++;
+  if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, fn, kargs);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    set_error("launch of %s failed: %s", what, cudaGetErrorString(e));
-    return RBFFD_ECUDA;
+    return false;
   }
-  return RBFFD_OK;
+  ctx->launches++;
+  return true;
 }
 
 }  // namespace rbffd

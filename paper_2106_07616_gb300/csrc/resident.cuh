@@ -80,9 +80,12 @@ ResPlan res_plan(rbffd_ctx *ctx, int n, int q);
 // Lists of a packed matrix's columns; longest list to *d_hmax (device).
 int res_halo_build(rbffd_ctx *ctx, const ResPlan &p, int n, int q, int ldn, const int32_t *col,
                    int32_t *hlist, int32_t *hinfo, uint16_t *lidx, int *d_hmax);
-// Launch fn(args) on the plan's team: a cooperative grid, or one cluster.
-int res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, size_t smem,
-               const char *what);
+// Launch fn(args) on the plan's team: a cooperative grid, or one cluster.  False
+// where the launch is refused -- a cluster of more than 8 CTAs or a CTA on every
+// SM may not be there to have -- and the solve has to stream; an error that is
+// no such refusal meets the streaming launch too, which reports it.  (Asking the
+// occupancy before each launch instead cost 8 to 15 us a launch.)
+bool res_launch(rbffd_ctx *ctx, const ResPlan &p, const void *fn, void *args, size_t smem);
 
 namespace res {
 
