@@ -131,16 +131,37 @@ __global__ void k_cell_count(int n, const double *__restrict__ x, const double *
   atomicAdd(&cnt[c], 1);
 }
 
+// The sum of each tile of KNN_TILE counts.
+constexpr int KNN_TILE = 1024;
+__global__ void __launch_bounds__(KNN_TILE) k_tile_sums(const int *__restrict__ cnt,
+                                                        int *__restrict__ sums, int m) {
+  __shared__ int s[32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, k = blockIdx.x * KNN_TILE + t;
+  int v = k < m ? cnt[k] : 0;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    v = s[lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) sums[blockIdx.x] = v;
+  }
+}
+
 // Exclusive scan of m counts, start[m] = total; a block a tile of 1024.  Each
-// block sums the counts before its tile itself (a coalesced read of at most
-// the whole array, from L2) instead of waiting for the block before it: one
-// block walking 75 000 counts took longer than the search of its points.
-__global__ void __launch_bounds__(1024) k_scan(const int *__restrict__ cnt,
-                                               int *__restrict__ start, int m) {
+// block sums what lies before its tile itself (a coalesced read, from L2)
+// instead of waiting for the block before it: one block walking 75 000 counts
+// took longer than the search of its points.  It reads the tiles' sums where
+// they were made (sums not null), else the counts.
+__global__ void __launch_bounds__(KNN_TILE) k_scan(const int *__restrict__ cnt,
+                                                   const int *__restrict__ sums,
+                                                   int *__restrict__ start, int m) {
   __shared__ int s[32], base_s;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, k0 = blockIdx.x * 1024;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, k0 = blockIdx.x * KNN_TILE;
+  const int *lead = sums != nullptr ? sums : cnt;
+  const int leads = sums != nullptr ? blockIdx.x : k0;
   int before = 0;
-  for (int k = t; k < k0; k += 1024) before += cnt[k];
+  for (int k = t; k < leads; k += KNN_TILE) before += lead[k];
   for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
   if (lane == 0) s[w] = before;
   __syncthreads();
@@ -428,6 +449,12 @@ __global__ void __launch_bounds__(128) k_knn_query(
   for (int s = 0; s < K; ++s) idx[o + 1 + s] = bj[s];
 }
 
+// Tiles above which their sums are made first: below, every block's own sum is
+// as fast as one launch more (150 000 points, 74 tiles: 273 us the whole call
+// either way; 300 000, 147 tiles: 500 and 497 us), above, it grows with the
+// square of the points (16 million: about 5 of 29 ms).
+constexpr int KNN_SUM_TILES = 128;
+
 int knn_workspace_bytes(int n, KnnLayout *lay) {
   int G = (int)ceil(sqrt((double)n / 2.0));
   if (G < 1) G = 1;
@@ -447,6 +474,7 @@ int knn_workspace_bytes(int n, KnnLayout *lay) {
   lay->off_grid = take(sizeof(Grid));
   lay->off_cell = take((size_t)n * sizeof(int));
   lay->off_start = take((size_t)(m + 1) * sizeof(int));
+  lay->off_sums = take((size_t)((m + KNN_TILE - 1) / KNN_TILE) * sizeof(int));
   lay->off_pts = take((size_t)n * sizeof(int));
   lay->bytes = off;
   return RBFFD_OK;
@@ -470,7 +498,14 @@ int knn_run(rbffd_ctx *ctx, void *ws, const KnnLayout &lay, int n, const double 
   RBFFD_TRY(after_launch(ctx, "k_bbox"));
   k_cell_count<<<nb, 256, 0, st>>>(n, x, y, bbox, m, cell, cnt, grid);
   RBFFD_TRY(after_launch(ctx, "k_cell_count"));
-  k_scan<<<(m + 1023) / 1024, 1024, 0, st>>>(cnt, start, m);
+  const int tiles = (m + KNN_TILE - 1) / KNN_TILE;
+  int *sums = nullptr;
+  if (tiles > KNN_SUM_TILES) {
+    sums = (int *)(b + lay.off_sums);
+    k_tile_sums<<<tiles, KNN_TILE, 0, st>>>(cnt, sums, m);
+    RBFFD_TRY(after_launch(ctx, "k_tile_sums"));
+  }
+  k_scan<<<tiles, KNN_TILE, 0, st>>>(cnt, sums, start, m);
   RBFFD_TRY(after_launch(ctx, "k_scan"));
   k_cell_fill<<<nb, 256, 0, st>>>(n, cell, start, cnt, pts);
   RBFFD_TRY(after_launch(ctx, "k_cell_fill"));

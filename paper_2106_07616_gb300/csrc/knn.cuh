@@ -8,7 +8,7 @@ namespace rbffd {
 
 struct KnnLayout {
   int m;              // cells at most
-  size_t off_bbox, off_cnt, off_grid, off_cell, off_start, off_pts;
+  size_t off_bbox, off_cnt, off_grid, off_cell, off_start, off_sums, off_pts;
   size_t zero_bytes;  // the first bytes, zeroed before a search
   size_t bytes;
 };

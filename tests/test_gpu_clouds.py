@@ -103,3 +103,22 @@ def test_a_long_line_takes_no_longer_than_a_square_cloud():
     square = seconds(*clouds.random_cloud(40000, 3))
     for x, y in (noisy_line(40000, 1e-15, 3), noisy_line(40000, 1e-15, 3)[::-1]):
         assert seconds(x, y) < 20 * square + 0.01
+
+
+@pytest.mark.parametrize("n", [262144, 263000, 600001])
+def test_many_cells_match_brute_force_on_a_sample(n):
+    """Around the number of cells from which the scan's tiles are summed first,
+    and well above: every point's cloud holds distinct points in order, and a
+    sample's clouds are the brute force's."""
+    g = torch.Generator(device="cuda:0").manual_seed(n)
+    x, y = (torch.rand(n, generator=g, device="cuda:0", dtype=torch.float64) for _ in range(2))
+    q = 12
+    idx = torch.zeros((n, q), dtype=torch.int32, device="cuda:0")
+    rbffd.rbffd_build_stencils(ctx(), x, y, None, q, idx)
+    c = idx.long()
+    assert torch.equal(c[:, 0], torch.arange(n, device="cuda:0"))
+    d2 = (x[c] - x[:, None]) ** 2 + (y[c] - y[:, None]) ** 2
+    assert bool((d2[:, 1:] > d2[:, :-1]).all())
+    for i in torch.randint(n, (64,), generator=g, device="cuda:0").tolist() + [0, n - 1]:
+        far = (x - x[i]) ** 2 + (y - y[i]) ** 2
+        assert torch.equal(torch.topk(far, q, largest=False).indices, c[i])
