@@ -45,3 +45,40 @@ def test_plan_teams_rejects_bad_input():
         rbffd.plan_teams([1.0], [0], [10], 4)
     with pytest.raises(rbffd.RbffdError):
         rbffd.plan_teams([-1.0], [1], [10], 4)
+
+
+def plain_search(work, cap, rows, cmax):
+    """The plan's span by a search that leaves nothing out."""
+    m, best = len(work), np.inf
+    order = np.argsort(-work, kind="stable")
+    g, gmax = 1, min(m, cmax)
+    while g <= gmax:
+        w, lat, most = np.zeros(g), np.zeros(g), np.full(g, 160)
+        for i in order:
+            k = int(np.argmin(w))
+            w[k] += work[i]
+            lat[k] += work[i] / rows[i] * LAT
+            most[k] = min(most[k], cap[i], max(1, (rows[i] * 8 + 255) // 256))
+        c, left = np.ones(g), cmax - g
+        while True:
+            k = int(np.argmax(lat + w / c))
+            if left == 0 or c[k] >= most[k]:
+                break
+            c[k] += 1
+            left -= 1
+        best = min(best, float((lat + w / c).max()))
+        g = gmax + 1 if g == gmax else min(gmax, g + max(1, g // 16))
+    return best
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_plan_teams_leaves_out_no_shorter_plan(seed):
+    """Counts of groups skipped by the bounds hold no shorter plan."""
+    _build.build()
+    rng = np.random.Generator(np.random.PCG64(seed))
+    m, cmax = int(rng.integers(1, 60)), int(rng.choice([60, 152, 304]))
+    rows = np.exp(rng.uniform(np.log(100), np.log(100 * 4 ** (1 + seed % 4)), m)).astype(np.int32)
+    work = rows * rng.integers(20, 150, m).astype(np.float64)
+    cap = np.minimum(160, np.maximum(1, rows // 60)).astype(np.int32)
+    *_, span = rbffd.plan_teams(work, cap, rows, cmax)
+    assert span == pytest.approx(plain_search(work, cap, rows, cmax), rel=1e-12)
