@@ -96,10 +96,12 @@ def solver_codes(args, rbffd):
 
 KRYLOV_PROFILES = {
     # preconditioner: (committed ncu summary, kernel sources it was taken from)
-    "jacobi": ("k_bicgstab_fp64_cavity200.md", ("krylov.cu", "krylov_dev.cuh", "common.cuh")),
-    "amg": ("k_bicgstab_amg_fp64_cavity200.md",
-            ("krylov.cu", "krylov_dev.cuh", "common.cuh", "amg_dev.cuh", "amg.cuh", "amg.cu",
-             "amg_setup.cu")),
+    "jacobi": ("k_bicg_res_jacobi_cavity200.md",
+               ("krylov_res.cu", "bicg_scalars.cuh", "resident.cu", "resident.cuh",
+                "common.cuh")),
+    "amg": ("k_bicg_res_amg_cavity200.md",
+            ("krylov_res.cu", "bicg_scalars.cuh", "resident.cu", "resident.cuh", "common.cuh",
+             "amg.cuh", "amg.cu", "amg_setup.cu")),
     "fgmres": ("k_fgmres_res_cavity200.md",
                ("fgmres_res.cu", "fgmres.cuh", "resident.cu", "resident.cuh", "common.cuh",
                 "amg.cuh", "amg.cu", "amg_setup.cu")),
@@ -686,14 +688,14 @@ def run_native(args):
             "peak_source": peak_src,
             "kernel": ("k_fgmres_res (pressure-correction flexible GMRES(30), FP32 multigrid "
                        "V-cycle preconditioner, persistent)" if args.precond == "fgmres" else
-                       "k_bicgstab_amg<1024> (pressure-correction BiCGSTAB, multigrid "
+                       "k_bicg_res<1, true> (pressure-correction BiCGSTAB, multigrid "
                        "V-cycle preconditioner, persistent)" if args.precond == "amg" and
                        args.precision == "fp64" else
-                       {"mixed": "k_bicgstab_ir<1> (pressure-correction FP32 BiCGSTAB in FP64 "
+                       {"mixed": "k_ir_res<1> (pressure-correction FP32 BiCGSTAB in FP64 "
                                 "refinement)",
-                       "ff": "k_bicgstab_ir<1> (pressure-correction float-float BiCGSTAB in "
+                       "ff": "k_ir_res<1> (pressure-correction float-float BiCGSTAB in "
                              "FP64 refinement)"}.get(
-                           args.precision, "k_bicgstab<1> (pressure-correction BiCGSTAB, persistent)")),
+                           args.precision, "k_bicg_res<1, false> (pressure-correction BiCGSTAB, persistent)")),
             "launches": kp["launches"], "avg_launch_ms": kp["ms"] / max(kp["launches"], 1),
             "bytes_per_unit": (f"q(4+4)+8 (FP32 SpMV) + one FP32 V-cycle + FP32 Gram-Schmidt "
                                f"over the basis per row-step (pcorr_bytes)"

@@ -355,7 +355,8 @@ struct ResCost {
 };
 constexpr ResCost RES_COST[2] = {{20.0, 0.002, 0.0013}, {38.0, 0.040, 0.0024}};
 // A unit of plan_by_time's spans (a row of a 256-thread CTA) in us per entry
-// of the row: launches of 16 members (q = 12 to 42) and of four (q = 20, 30).
+// of the row: fitted to launches of 16 members (q = 12 to 42) and of four (q = 20,
+// 30); nothing between or beyond them was measured.
 constexpr double STREAM_UNIT[2] = {0.0020, 0.0052};
 
 // Members of more rows in all than this (half of what a chip of 1024-thread

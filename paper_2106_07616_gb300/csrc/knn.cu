@@ -208,9 +208,10 @@ __device__ __forceinline__ bool key_less(double da, int ja, double db, int jb) {
 // local memory.  A thread with an insertion-sorted list per point was bound
 // by that list's local-memory traffic and by divergence: the whole search of
 // 147 827 graded points at q = 20 took 1.20 ms with it, 0.55 ms this way, and
-// 0.41 ms with the ranks counted by d^2 alone (the index decides only where a
-// place stays empty), two candidates a lane at once, and the grid's FP64
-// divisions made once instead of by every block of four points.  It is bound
+// 0.40 ms with the ranks counted by d^2 alone (the index decides only where a
+// place stays empty), two candidates a lane at once, the grid's FP64 divisions
+// made once instead of by every block of four points, and the block's limit
+// one product.  It is bound
 // by instruction issue and the FP64 distances (53% of the pipe before).
 // Points whose block holds more than CAP candidates at every usable r go to
 // the list `rest` (k_knn_query searches them).

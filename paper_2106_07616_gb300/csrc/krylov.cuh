@@ -106,7 +106,11 @@ int krylov_launch(rbffd_ctx *ctx, int nr, int nblocks, const KrylovArgs &args);
 // The same solve on a resident team (krylov_res.cu), when the plan, the sizes
 // and, with a multigrid preconditioner, its hierarchy h allow it (*ran);
 // omega: level 0's smoothing weight; B: the dense coarse operator or null.
-constexpr int RES_DENSE64_N = 512;  // most level-1 rows of an FP64 dense coarse operator
+// Most level-1 rows of an FP64 dense coarse operator: 2 MB a problem.  Faster than
+// the composed cycle's two phases at every size measured: outer iterations with
+// and without it 2.57 and 2.90 ms at 119 rows, 4.28 and 4.57 at 479; above the
+// limit 4.20 and 4.67 at 638, 3.43 and 3.94 at 1 082, 4.63 and 4.71 at 1 453 (17 MB).
+constexpr int RES_DENSE64_N = 512;
 int krylov_res_launch(rbffd_ctx *ctx, int nr, const KrylovArgs &args, const AmgDev *h,
                       double omega, const double *B, bool *ran);
 // Batched: args.res holds the team (nb, R, hmax; hlist null: the kernel makes

@@ -28,7 +28,12 @@ namespace rbffd {
 constexpr int RES_NT = 1024;        // threads per CTA of a resident solve
 constexpr int RES_MAXB = 160;       // CTAs of a team
 constexpr int RES_CLUSTER = 16;     // most CTAs of a cluster team
-constexpr int RES_CLUSTER_N = 4096; // most rows of a cluster team
+// Most rows of a cluster team: where the FP64 solves stop gaining.  Outer
+// iterations on Kovasznay lattices, cluster and grid, ms: 4 096 rows mixed 2.22
+// and 2.80, FP64 multigrid 4.05 and 4.36, FP64 Jacobi 10.1 and 11.2 (900 rows: 1.8
+// and 2.4, 2.8 and 3.3, 4.3 and 5.0); 5 184 rows mixed 2.67 and 2.93, FP64 5.20 and
+// 4.58; 10 000 rows 3.40 and 2.97, 6.90 and 4.62.
+constexpr int RES_CLUSTER_N = 4096;
 constexpr int RES_HCAP = 8192;      // largest halo list (16-bit byte offsets of 8-byte entries)
 constexpr int RES_MAXN = 150 * RES_NT;  // rows a team can own, one lane each
 // Most dynamic shared memory of a resident launch.  Every launch allows its

@@ -1,7 +1,8 @@
-// weights.cu -- S2: PHS r^3 + polynomial collocation weights, 4 to 32 lanes a
-// cloud, the augmented (q+m) x (q+m+3) system in shared memory, FP64 LU with
-// partial pivoting (paper Sec. 2, Eqs. RBF_interp_mat_vec ..
-// RBF_interp_mat_vec_L_solve).
+// weights.cu -- S2: PHS r^3 + polynomial collocation weights (paper Sec. 2, Eqs.
+// RBF_interp_mat_vec .. RBF_interp_mat_vec_L_solve), 4 to 32 lanes a cloud: the
+// polynomials' factors and Phi with three right-hand sides in shared memory,
+// FP64 LU with partial pivoting of the polynomials (q x m) and of Phi on their
+// null space (q - m).
 //
 // The matrix build uses explicit round-to-nearest intrinsics (no fused
 // multiply-add), as the oracle does.  On GB300 the kernel is bound by the
@@ -24,11 +25,16 @@
 // augmented matrix, 3.2 ms by the null space with a warp a cloud and 16 warps a
 // block, 2.5 ms now: some 1 200 FP64 instructions a cloud, 19 000 cycles, keep
 // the pipe busy (89% of its cycles); 10 201 clouds at q = 12, degree 2 in 0.47,
-// 0.25 and 0.11 ms.  Relative error against 80-bit elimination, augmented and
-// null space, worst of the three operators: degree 2 8.9e-15 and 7.8e-15,
-// degree 3 3.9e-14 and 4.4e-14, degree 4 1.1e-13 and 1.3e-13 (graded cylinder
-// 6.5e-14 and 9.3e-14), degree 5 4.1e-13 and 4.0e-13; 64-bit elimination with
-// another order of its sums lies as far apart (1.4e-13 at degree 4).
+// 0.25 and 0.11 ms.  Relative error against 80-bit elimination over 800 clouds
+// each, this kernel, the augmented elimination before it and an unfused one (d/dx,
+// d/dy, Laplacian): degree 2 7.5e-15 7.5e-15 5.1e-15, 8.5e-15 8.8e-15 6.2e-15,
+// 8.7e-15 8.6e-15 6.2e-15; degree 3 4.7e-14 4.5e-14 2.5e-14, 3.9e-14 3.9e-14
+// 2.4e-14, 4.1e-14 3.9e-14 2.4e-14; degree 4 0.96e-13 1.24e-13 5.7e-14, 0.96e-13
+// 0.93e-13 4.8e-14, 1.17e-13 1.02e-13 4.8e-14 (graded cylinder 8.3e-14 7.8e-14
+// 3.5e-14, 5.9e-14 5.9e-14 3.0e-14, 6.3e-14 6.9e-14 2.9e-14); degree 5 3.8e-13
+// 4.1e-13 1.6e-13, 5.9e-13 5.7e-13 1.4e-13, 7.0e-13 7.9e-13 1.5e-13: up to 1.4
+// times the augmented elimination's, and below it in some.  It comes from the
+// rounding of Phi's entries and of the sums that form S: with both exact 3e-16.
 #include "abi_guard.cuh"
 #include "common.cuh"
 #include "weights.cuh"
