@@ -125,6 +125,18 @@ const char *rbffd_last_error(void);
 /* Number of kernel launches this context has issued (for accounting). */
 int64_t rbffd_ctx_launch_count(const rbffd_ctx *ctx);
 
+/* Bound of every device-side wait (the grid exchanges and barriers of the
+ * persistent Krylov kernels) of the launches this context issues from now
+ * on: 2^log2_cycles SM clock cycles; 0 restores the default 2^31 (about a
+ * second at 2 GHz).  A wait that runs out makes its block record a timeout
+ * and leave; the other blocks leave at their next wait, and the call returns
+ * RBFFD_ETIMEOUT with the solve's outputs unspecified.  Nothing is left
+ * running and the context stays usable.  Solves of one thread-block cluster
+ * (small problems) wait at the hardware's barrier, which has no limit and needs
+ * none: its blocks are resident together.  The paper has no counterpart: this
+ * is failure handling of the library.  Errors: RBFFD_EINVAL outside 0..40. */
+int rbffd_ctx_set_wait_limit(rbffd_ctx *ctx, int32_t log2_cycles);
+
 /* Live per-kernel timing.  While enabled, the context brackets the launches
  * of the classes below with CUDA events on its own stream (the stream the
  * kernels run on) and accumulates, per class: launches, device time, the
@@ -135,7 +147,8 @@ int64_t rbffd_ctx_launch_count(const rbffd_ctx *ctx);
  *   KRYLOV_MOM  (momentum BiCGSTAB, 2 right-hand sides sharing the matrix):
  *               unit = one row in one iteration; bytes = 2q(s_w + s_i) + 28 s_v
  *   WEIGHTS     unit = one cloud; "bytes" holds FP64 flops: 2N^3/3 + 2 N^2 (3 rhs)
- *               + the matrix build, N = q + m
+ *               + the matrix build, N = q + m (of the augmented elimination;
+ *               the kernel's null space takes about half)
  *   KNN         unit = one point; bytes = 24 (coordinates in, q indices out)
  *   OUTER       one outer iteration (whole simple_iterate, GPU time)
  * s_w, s_i, s_v: bytes of a matrix value, a column index, a vector entry
@@ -155,17 +168,7 @@ typedef struct {
   int64_t launches;
   double ms;     /* summed device time */
   double units;  /* units of work processed */
-  double bytes;  /* Bound of every device-side wait (the grid exchanges and barriers of the
- * persistent Krylov kernels) of the launches this context issues from now
- * on: 2^log2_cycles SM clock cycles; 0 restores the default 2^31 (about a
- * second at 2 GHz).  A wait that runs out makes its block record a timeout
- * and leave; the other blocks leave at their next wait, and the call returns
- * RBFFD_ETIMEOUT with the solve's outputs unspecified.  Nothing is left
- * running and the context stays usable.  The paper has no counterpart: this
- * is failure handling of the library.  Errors: RBFFD_EINVAL outside 0..40. */
-int rbffd_ctx_set_wait_limit(rbffd_ctx *ctx, int32_t log2_cycles);
-
-/* algorithmic bytes (flops for WEIGHTS) */
+  double bytes;  /* algorithmic bytes (flops for WEIGHTS) */
 } rbffd_kernel_stat;
 int rbffd_ctx_profile(rbffd_ctx *ctx, int enable);
 int rbffd_ctx_kernel_stat(const rbffd_ctx *ctx, int32_t which, rbffd_kernel_stat *out);

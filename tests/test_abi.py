@@ -77,3 +77,10 @@ print(rc, L.rbffd_last_error().decode())
     assert r.returncode == 0, r.stderr
     rc, _, text = r.stdout.strip().splitlines()[-1].partition(" ")
     assert int(rc) == -2 and "host resources exhausted" in text, r.stdout
+
+
+@pytest.mark.parametrize("lang", ["c", "c++"])
+def test_header_compiles_in_c_and_cpp(lang):
+    import subprocess
+    subprocess.run(["gcc", "-fsyntax-only", "-Wall", "-Werror", "-x", lang,
+                    os.path.join(ROOT, "include", "rbffd.h")], check=True)
